@@ -96,7 +96,13 @@ typedef struct {
                                  writes the next sweep's shares; a forward sweep also reduces
                                  the previous iteration's bound), two kernels per iteration.
                                  0: separate pending-sum kernels, four per iteration.  -1
-                                 (default): 0, the faster plan on every workload measured.
+                                 (default): plain solvers (alpha = 0, no split, averaging 0)
+                                 whose layout is left to the library too (lanes != 0, staging and
+                                 tune_layout not forced on, no layout_classes) and whose BDDs have
+                                 layers of at most two nodes and at most 32 of them run the
+                                 direct plan: every sweep forms the shares from the recorded
+                                 differences itself and recomputes the messages it needs, two
+                                 kernels per iteration; the others as 0.
                                  Same arithmetic either way: multipliers and pending sums are
                                  bit-identical; bounds differ only in the FP64 summation
                                  order. */

@@ -20,7 +20,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libbdd_dbca.so")
 LIB_CHECKED = os.path.join(BUILD, "libbdd_dbca_checked.so")
-SOURCES = ["compile.cpp", "order.cpp", "kernels.cu", "adjoint.cu", "api.cu", "noalloc.cu"]
+SOURCES = ["compile.cpp", "order.cpp", "kernels.cu", "direct.cu", "adjoint.cu", "api.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "nvcc")
 
@@ -33,7 +33,7 @@ def _inputs():
     return files
 
 
-CHECKED = "kernels.cu"  # the unit whose index checks -DBDD_CHECKED turns on
+CHECKED = ("kernels.cu", "direct.cu")  # the units whose index checks -DBDD_CHECKED turns on
 
 
 def _stale() -> bool:
@@ -76,13 +76,13 @@ def build(force: bool = False) -> str:
     if not force and not _stale():
         return LIB
     os.makedirs(BUILD, exist_ok=True)
-    jobs = [(src, False) for src in SOURCES] + [(CHECKED, True)]
+    jobs = [(src, False) for src in SOURCES] + [(src, True) for src in CHECKED]
     # the longest units first, so the parallel build ends with the short ones
     jobs.sort(key=lambda j: (not j[0].startswith("kernels"), j[0]))
     with cf.ThreadPoolExecutor(len(jobs)) as ex:
         objs = dict(zip(jobs, ex.map(_compile, jobs)))
     normal = [objs[(src, False)] for src in SOURCES]
-    checked = [objs[(src, src == CHECKED)] for src in SOURCES]
+    checked = [objs[(src, src in CHECKED)] for src in SOURCES]
     _link(LIB, normal)
     _link(LIB_CHECKED, checked)
     return LIB

@@ -156,6 +156,18 @@ struct bdd_solver {
   int4 *d_cut_grp = nullptr, *d_pair = nullptr;
   int *d_head_node = nullptr, *d_head_ptr = nullptr, *d_head_pair = nullptr;
   float *d_mu_bar = nullptr, *d_mu = nullptr, *d_dfwd = nullptr, *d_dbwd = nullptr;
+  // direct plan (DirectLayout in internal.h)
+  bool direct = false;
+  DirectLayout dlayout;          // kept in host memory for host_only == 2 only
+  long long Od = 0, ext = 0;     // occurrences with padding, grouped values
+  int n_tiles = 0, deep_depth = 0, chains = 0, n_coop = 0, warp_depth = 0, heavy0 = 0, grid_direct = 0;
+  size_t smem_direct = 0;
+  int4 *d_tile = nullptr;
+  int *d_ref = nullptr, *d_home = nullptr, *d_heavy_of = nullptr;
+  unsigned char *d_ext_deg = nullptr;
+  float *d_diff_f = nullptr, *d_diff_b = nullptr;  // differences of the last forward / backward sweep
+  float2 *d_heavy_sum = nullptr;
+  double *d_const = nullptr;     // empty_const, read by the captured reductions
   cudaEvent_t ev_last = nullptr;  // end of the solver's last enqueued work, on whatever stream
 
   bdd_solver() {
@@ -252,6 +264,80 @@ struct bdd_solver {
     c.gamma = gamma;
     c.ngroups = npairs > 0 ? (int)ngroups : 0;
     return c;
+  }
+
+  // a sweep of the direct plan: a forward sweep reads the differences of the backward sweep before
+  // it and writes its own, a backward sweep the other way round
+  DirectParams direct_params(bool fwd) const {
+    DirectParams p{};
+    p.tile = d_tile;
+    p.n_tiles = n_tiles;
+    p.code = d_lane_code;
+    p.ref = d_ref;
+    p.csr = d_occ_csr;
+    p.lam = d_lam;
+    p.din = fwd ? d_diff_b : d_diff_f;
+    p.dout = fwd ? d_diff_f : d_diff_b;
+    p.ein = p.din + Od;
+    p.ext_deg = d_ext_deg;
+    p.heavy_of = d_heavy_of;
+    p.heavy = d_heavy_sum;
+    p.heavy0 = heavy0;
+    p.deep_depth = deep_depth;
+    p.chains = chains;
+    p.n_coop = n_coop;
+    p.warp_depth = warp_depth;
+    p.omega = omega;
+    p.bdd_E = d_bdd_E;
+    p.partial = d_partial;
+    p.error = d_error;
+    p.n_diff = Od + ext;
+    p.n_csr = nnz;
+    p.n_bdd = nb;
+    p.n_occ = Od;
+    p.fin_nblocks = grid_direct;
+    p.iter_ctr = d_iter;
+    p.trace = d_trace;
+    p.trace_cap = trace_cap;
+    p.empty_const = d_const;
+    p.ticket = d_ticket;
+    p.pdl_early = pdl_early ? 1 : 0;
+    return p;
+  }
+  // sum_bound: a forward sweep adds up the bound of the iteration before, the backward sweep after
+  // it finishes that sum
+  int direct_sweep(bool fwd, bool sum_bound, cudaStream_t s) {
+    DirectParams p = direct_params(fwd);
+    if (fwd) p.sum_bound = sum_bound ? 1 : 0;
+    else p.fin_partial = sum_bound ? d_partial : nullptr;
+    if (direct_launch(fwd, kDirectUpdate, p, grid_direct, smem_direct, s)) return BDD_ECUDA;
+    return direct_heavy(fwd, s);
+  }
+  int direct_heavy(bool fwd, cudaStream_t s) {
+    return heavy_launch(d_heavy, n_heavy, (fwd ? d_diff_f : d_diff_b) + Od, d_heavy_sum, s) ? BDD_ECUDA : BDD_OK;
+  }
+  // E^j of the current multipliers; with sum_bound also the bound into the trace
+  int direct_energy(bool sum_bound, cudaStream_t s) {
+    DirectParams p = direct_params(true);
+    p.sum_bound = sum_bound ? 1 : 0;
+    return direct_launch(true, kDirectEnergy, p, grid_direct, smem_direct, s) ? BDD_ECUDA : BDD_OK;
+  }
+  // the constant of the variables in no row, where the captured reductions read it
+  int put_const(cudaStream_t s) {
+    if (d_const) CK(cudaMemcpyAsync(d_const, &empty_const, sizeof(double), cudaMemcpyHostToDevice, s));
+    return BDD_OK;
+  }
+  // the pending sums, which the direct plan keeps as differences only
+  int direct_pending(cudaStream_t s) {
+    return direct_pending_launch(d_home, d_ref, d_var_ptr, d_diff_b, Od, d_P, n, s) ? BDD_ECUDA : BDD_OK;
+  }
+  int direct_restart(cudaStream_t s) {
+    if (direct_init_launch(d_occ_var, d_var_ptr, d_c, d_lam, Od, s)) return BDD_ECUDA;
+    const size_t db = sizeof(float) * (size_t)std::max<long long>(Od + ext, 1);
+    CK(cudaMemsetAsync(d_diff_f, 0, db, s));
+    CK(cudaMemsetAsync(d_diff_b, 0, db, s));
+    RC(direct_heavy(false, s));
+    return direct_energy(false, s);
   }
 
   // copy-arc dual step after a sweep (split solvers; nothing otherwise)
@@ -412,6 +498,11 @@ struct bdd_solver {
   // plan: forward sweep (reducing the previous iteration's bound unless `first`), backward
   // sweep, and with `last` the bound kernel.
   int enqueue_iteration(cudaStream_t s, bool first = true, bool last = true) {
+    if (direct) {
+      RC(direct_sweep(true, !first, s));
+      RC(direct_sweep(false, !first, s));
+      return last ? direct_energy(true, s) : BDD_OK;
+    }
     if (fused) {
       if (sweep_launch(true, kUpdateFused, fused_params(!first), grid_sweep, s)) return BDD_ECUDA;
       if (sweep_launch(false, kUpdateFused, fused_params(false), grid_sweep, s)) return BDD_ECUDA;
@@ -515,6 +606,7 @@ struct bdd_solver {
   // lambda^j_i = c_i/|J_i|, P = 0, then backward messages (and E^j) for that lambda.  Split
   // solvers: copy-arc duals and their last deltas 0, so every root message is 0.
   int restart(cudaStream_t s) {
+    if (direct) return direct_restart(s);
     if (O > 0 && init_lambda_launch(d_occ_var, d_var_ptr, d_c, d_lam, (int)O, s)) return BDD_ECUDA;
     if (npairs > 0) {
       const size_t pb = sizeof(float) * (size_t)npairs;
@@ -533,6 +625,24 @@ struct bdd_solver {
   // min-marginals and folded multipliers for the current state; leaves the state unchanged
   int output_pass(cudaStream_t s, float *lam_out, float *m0, float *m1) {
     const size_t bytes = sizeof(float) * (size_t)nnz;
+    if (direct) {
+      if (lam_out) {
+        if (nnz > O) CK(cudaMemsetAsync(lam_out, 0, bytes, s));
+        if (direct_scatter_launch(direct_params(true), Od, lam_out, true, s)) return BDD_ECUDA;
+      }
+      if (m0 || m1) {
+        if (!m0 || !m1) RC(ensure_outputs());
+        DirectParams p = direct_params(true);
+        p.out_m0 = m0 ? m0 : d_out_m0;
+        p.out_m1 = m1 ? m1 : d_out_m1;
+        if (nnz > O) {  // zero coefficients have no occurrence
+          CK(cudaMemsetAsync(p.out_m0, 0, bytes, s));
+          CK(cudaMemsetAsync(p.out_m1, 0, bytes, s));
+        }
+        if (direct_launch(true, kDirectFolded, p, grid_direct, smem_direct, s)) return BDD_ECUDA;
+      }
+      return BDD_OK;
+    }
     if (lam_out) {
       if (nnz) CK(cudaMemsetAsync(lam_out, 0, bytes, s));
       if (O && scatter_lambda_launch(d_lam, d_share_occ, d_occ_csr, lam_out, (int)O, true, s))
@@ -786,6 +896,93 @@ int setup_device(bdd_solver *h, const Layout &L, const float *c, const CutTables
   return BDD_OK;
 }
 
+int setup_direct(bdd_solver *h, const DirectLayout &L, const float *c) {
+  CK(cudaEventCreateWithFlags(&h->ev_last, cudaEventDisableTiming));
+  h->direct = true;
+  h->bdd_perm = L.bdd_perm;
+  for (int t = 0; t < kWarpClasses + 2; ++t) h->class_tile_off[t] = L.class_tile_off[t];
+  h->n_tiles = L.n_tiles;
+  h->n_warp_tiles = L.n_tiles;
+  h->deep_depth = L.deep_depth;
+  h->chains = L.chains ? 1 : 0;
+  h->Od = L.Od;
+  h->ext = L.ext;
+  h->heavy0 = (int)L.heavy0;
+  const long long n = h->n, nb = h->nb, Od = h->Od, D = h->Od + h->ext;
+  int dev = 0, nsm = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return BDD_ECUDA;
+  // deep tiles of more than kCoopDepth layers take a block each, whose warps share the loads of the
+  // layers, as long as there are at most as many as SMs (300x300 matching, 19 such tiles: a sweep of
+  // 31 us with a warp to a tile, 16 with a block, 12.5 once the walks read a layer ahead); more of
+  // them fill the GPU with a warp each
+  h->warp_depth = h->deep_depth;
+  if (h->deep_depth > kCoopDepth) {
+    int coop = 0;
+    while (coop < L.n_tiles && (L.tile[4 * coop + 3] & kTileDepth) > kCoopDepth && (L.tile[4 * coop + 2] & kTileDeep)) ++coop;
+    const bool all = coop == L.n_tiles || (L.tile[4 * coop + 3] & kTileDepth) <= kCoopDepth;
+    if (coop <= nsm && all) {
+      h->n_coop = coop;
+      h->warp_depth = std::min(h->deep_depth, kCoopDepth);
+    }
+  }
+  h->smem_direct = (size_t)kLaneLayerBytes * std::max(kWarpsPerBlock * h->warp_depth, h->n_coop ? h->deep_depth : 0);
+  if (h->smem_direct > 48 * 1024 && direct_set_smem(h->smem_direct)) return BDD_ECUDA;
+  if (direct_resident_blocks(L.chains, h->smem_direct, &per_sm)) return BDD_ECUDA;
+  // one wave of blocks at most: the warps take the tiles in turn (deepest first), so the bound has
+  // one partial per resident block and every block but the first few lives as long as the sweep
+  const int wave = std::max(1, nsm) * std::max(1, per_sm);
+  h->grid_direct = h->n_coop + std::max(1, std::min((L.n_tiles - h->n_coop + kWarpsPerBlock - 1) / kWarpsPerBlock, wave - h->n_coop));
+  h->pdl_early = h->grid_direct < wave;
+  const long long need = 29 * Od + 12 * h->ext + 4 * (3 * n + 1) + 12 * nb + 16LL * L.n_tiles + 8LL * h->grid_direct + 1024 * 8;
+  if (h->max_device_bytes > 0 && need > h->max_device_bytes) return BDD_ENOMEM;
+  {
+    int *tmp = nullptr;
+    RC(upload(h, &tmp, L.tile));
+    h->d_tile = reinterpret_cast<int4 *>(tmp);
+    tmp = nullptr;
+    RC(upload(h, &tmp, L.heavy));
+    h->d_heavy = reinterpret_cast<int4 *>(tmp);
+    h->n_heavy = (int)(L.heavy.size() / 4);
+  }
+  RC(upload(h, &h->d_lane_code, L.code));
+  RC(upload(h, &h->d_ref, L.ref));
+  RC(upload(h, &h->d_occ_csr, L.csr));
+  RC(upload(h, &h->d_occ_var, L.var));
+  RC(upload(h, &h->d_home, L.home));
+  RC(upload(h, &h->d_var_ptr, L.var_ptr));
+  RC(upload(h, &h->d_ext_deg, L.ext_deg));
+  RC(upload(h, &h->d_heavy_of, L.heavy_of));
+  RC(upload(h, &h->d_bdd_depth, L.bdd_depth));
+  {
+    std::vector<int> rows(nb);
+    for (long long t = 0; t < nb; ++t) rows[t] = h->canon_row[L.bdd_perm[t]];
+    RC(upload(h, &h->d_bdd_row, rows));
+  }
+  RC(h->alloc(&h->d_lam, Od));
+  RC(h->alloc(&h->d_diff_f, D));
+  RC(h->alloc(&h->d_diff_b, D));
+  RC(h->alloc(&h->d_heavy_sum, h->n_heavy));
+  RC(h->alloc(&h->d_P, n));
+  RC(h->alloc(&h->d_c, n));
+  RC(h->alloc(&h->d_bdd_E, nb));
+  RC(h->alloc(&h->d_partial, h->grid_direct));
+  RC(h->alloc(&h->d_error, 1));
+  RC(h->alloc(&h->d_ticket, 1));
+  RC(h->alloc(&h->d_iter, 1));
+  RC(h->alloc(&h->d_const, 1));
+  CK(cudaMemset(h->d_error, 0, sizeof(int)));
+  CK(cudaMemset(h->d_ticket, 0, sizeof(unsigned)));
+  CK(cudaMemset(h->d_iter, 0, sizeof(int)));
+  RC(h->ensure_trace(1024));
+  if (n) CK(cudaMemcpy(h->d_c, c, sizeof(float) * n, cudaMemcpyHostToDevice));
+  RC(h->put_const(h->stream));
+  RC(h->restart(h->stream));
+  RC(h->end(h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  return BDD_OK;
+}
+
 // ---------------------------------------------------------------------------------------
 // Layout tuner.  Each key (a BDD's natural width class and its depth bucket) has up to two tile
 // classes its BDDs can run in: lane tiles or two-lane teams for widths <= 2; a team of 2^c or of
@@ -971,6 +1168,112 @@ double empty_constant(const std::vector<int> &deg, const float *c, int n, double
   return s;
 }
 
+// canonical form from the direct layout's lane codes (bdd_export_canonical)
+int export_direct(const bdd_solver *h, int *bdd_row, int *bdd_depth, int *occ_var, long long *occ_csr, int *occ_width,
+                  int *lo, int *hi) {
+  const long long nb = h->nb, O = h->O, N = h->N;
+  DirectLayout read;
+  const DirectLayout &L = h->host_layout ? h->dlayout : read;
+  if (!h->host_layout) {
+    DeviceGuard dg(h->device);
+    if (!dg.ok) return BDD_ECUDA;
+    read.tile.resize(4 * (size_t)h->n_tiles);
+    read.bdd_depth.resize(nb);
+    read.code.resize(h->Od);
+    read.var.resize(h->Od);
+    read.csr.resize(h->Od);
+    CK(cudaEventSynchronize(h->ev_last));
+    if (h->n_tiles) CK(cudaMemcpy(read.tile.data(), h->d_tile, sizeof(int4) * h->n_tiles, cudaMemcpyDeviceToHost));
+    if (nb) CK(cudaMemcpy(read.bdd_depth.data(), h->d_bdd_depth, sizeof(int) * nb, cudaMemcpyDeviceToHost));
+    if (h->Od) {
+      CK(cudaMemcpy(read.code.data(), h->d_lane_code, h->Od, cudaMemcpyDeviceToHost));
+      CK(cudaMemcpy(read.var.data(), h->d_occ_var, sizeof(int) * h->Od, cudaMemcpyDeviceToHost));
+      CK(cudaMemcpy(read.csr.data(), h->d_occ_csr, sizeof(long long) * h->Od, cudaMemcpyDeviceToHost));
+    }
+  }
+  std::vector<int> sorted_of_canon(nb), tile_of(nb, -1);
+  for (long long s = 0; s < nb; ++s) sorted_of_canon[h->bdd_perm[s]] = (int)s;
+  for (int t = 0; t < h->n_warp_tiles; ++t)
+    for (int q = 0; q < (L.tile[4 * t + 2] & (kTileDeep - 1)); ++q)
+      if (L.tile[4 * t + 1] + q < nb) tile_of[L.tile[4 * t + 1] + q] = t;
+  long long co = 0, cn = 0;
+  for (long long cb = 0; cb < nb; ++cb) {
+    const int s = sorted_of_canon[cb], t = tile_of[s], depth = L.bdd_depth[s];
+    if (t < 0) return BDD_EDEVICE;
+    const int lane = s - L.tile[4 * t + 1];
+    bdd_row[cb] = h->canon_row[cb];
+    bdd_depth[cb] = depth;
+    if (lane > 31 || depth > (L.tile[4 * t + 3] & kTileDepth)) return BDD_EDEVICE;
+    for (int l = 0; l < depth; ++l, ++co) {
+      const long long o = L.tile[4 * t] + 32LL * l + lane;
+      if (co >= O) return BDD_EDEVICE;
+      const unsigned c = L.code[o];
+      const int w = (c >> 4) == (kDirectNoNode1 >> 4) ? 1 : 2;
+      occ_var[co] = L.var[o];
+      occ_csr[co] = L.csr[o];
+      occ_width[co] = w;
+      for (int q = 0; q < w; ++q, ++cn) {
+        if (cn >= N) return BDD_EDEVICE;
+        const unsigned a0 = (c >> (4 * q)) & 3u, a1 = (c >> (4 * q + 2)) & 3u;
+        const int node0 = l + 1 == depth ? kTop : 0;
+        lo[cn] = a0 == 0 ? node0 : a0 == kDirectBot ? kBot : (int)a0;
+        hi[cn] = a1 == 0 ? node0 : a1 == kDirectBot ? kBot : (int)a1;
+      }
+    }
+  }
+  return co == O && cn == N ? BDD_OK : BDD_EDEVICE;
+}
+
+// the device part of a build: device, streams, then `setup`
+template <class Setup>
+int on_device(bdd_solver *h, const bdd_options &opt, bdd_solver **out, Setup setup) {
+  int rc = BDD_OK;
+  {
+    DeviceGuard dg(opt.device);
+    if (!dg.ok) {
+      delete h;
+      return BDD_ECUDA;
+    }
+    cudaGetDevice(&h->device);
+    if (opt.stream) {
+      h->stream = (cudaStream_t)opt.stream;
+    } else if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaGetLastError();
+      delete h;
+      return BDD_ECUDA;
+    } else {
+      h->own_stream = true;
+    }
+    if (cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaGetLastError();
+      delete h;
+      return BDD_ECUDA;
+    }
+    rc = setup();
+    if (rc != BDD_OK) delete h;
+  }
+  if (rc == BDD_OK) *out = h;
+  return rc;
+}
+
+// a build whose direct layout is in h->dlayout
+int finish_build(bdd_solver *h, const bdd_options &opt, const float *c, bdd_solver **out) {
+  const DirectLayout &L = h->dlayout;
+  h->direct = true;
+  if (h->host_layout) {
+    h->bdd_perm = L.bdd_perm;
+    h->n_warp_tiles = L.n_tiles;
+    *out = h;
+    return BDD_OK;
+  }
+  h->host = HostBDDs();
+  return on_device(h, opt, out, [&]() {
+    const int rc = setup_direct(h, L, c);
+    h->dlayout = DirectLayout();
+    return rc;
+  });
+}
+
 }  // namespace
 
 extern "C" {
@@ -1144,6 +1447,31 @@ int bdd_build(int n, int m, const long long *row_ptr, const int *col, const int 
     *out = h;
     return BDD_OK;
   }
+  // the direct plan: plain solvers whose options leave the choice of layout and schedule to the
+  // library (its sweeps have one way to stage a tile and no pending pass to place)
+  if (plain && opt.averaging == 0 && opt.fused_pending == -1 && opt.staging == -1 && opt.lanes != 0 &&
+      !opt.layout_classes && opt.tune_layout != 1) {
+    DirectLayout &L = h->dlayout;
+    try {
+      rc = build_direct_layout(H, &L, h->var_deg.data());
+    } catch (const std::bad_alloc &) {
+      rc = BDD_ENOMEM;
+    }
+    if (rc == BDD_OK) {
+      h->lanes2 = L.class_tile_off[1] > 0;
+      bdd_keys(H, h->key_nodes);
+      for (int k = 0; k < 2 * kDepthBuckets; ++k) h->key_class[k] = h->key_nodes[k] ? 0 : -1;
+      h->lane_O = h->O;
+      h->lane_N = h->N;
+      return finish_build(h, opt, c, out);
+    }
+    L = DirectLayout();
+    if (rc != BDD_ETOOBIG) {
+      delete h;
+      return rc;
+    }
+    rc = BDD_OK;
+  }
   // tile class of every layout key: explicit, tuned on the device, or the defaults
   bool keyed = false;
   if (opt.layout_classes) {
@@ -1207,35 +1535,7 @@ int bdd_build(int n, int m, const long long *row_ptr, const int *col, const int 
     return BDD_OK;
   }
   H = HostBDDs();  // the device slabs are the only copy from here on
-  {
-    DeviceGuard dg(opt.device);
-    if (!dg.ok) {
-      delete h;
-      return BDD_ECUDA;
-    }
-    cudaGetDevice(&h->device);
-    if (opt.stream) {
-      h->stream = (cudaStream_t)opt.stream;
-    } else if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess) {
-      cudaGetLastError();
-      delete h;
-      return BDD_ECUDA;
-    } else {
-      h->own_stream = true;
-    }
-    if (cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
-      cudaGetLastError();
-      delete h;
-      return BDD_ECUDA;
-    }
-    rc = setup_device(h, L, c, ct);
-  }
-  if (rc != BDD_OK) {
-    delete h;
-    return rc;
-  }
-  *out = h;
-  return BDD_OK;
+  return on_device(h, opt, out, [&]() { return setup_device(h, L, c, ct); });
 }
 
 int bdd_iterate_device(bdd_solver *h, int n_iter, double *d_bound_trace, float *d_lambda, float *d_mm0,
@@ -1300,6 +1600,16 @@ int bdd_iterate_profiled(bdd_solver *h, int n_iter, double *kernel_ms) {
         if (rc == BDD_OK && cudaEventRecord(e[4], s) != cudaSuccess) rc = BDD_ECUDA;
         continue;
       }
+      if (h->direct) {  // forward sweep, (heavy variables with it), backward sweep, bound
+        if (rc == BDD_OK) rc = h->direct_sweep(true, false, s);
+        if (rc == BDD_OK && cudaEventRecord(e[1], s) != cudaSuccess) rc = BDD_ECUDA;
+        if (rc == BDD_OK && cudaEventRecord(e[2], s) != cudaSuccess) rc = BDD_ECUDA;
+        if (rc == BDD_OK) rc = h->direct_sweep(false, false, s);
+        if (rc == BDD_OK && cudaEventRecord(e[3], s) != cudaSuccess) rc = BDD_ECUDA;
+        if (rc == BDD_OK) rc = h->direct_energy(true, s);
+        if (rc == BDD_OK && cudaEventRecord(e[4], s) != cudaSuccess) rc = BDD_ECUDA;
+        continue;
+      }
       if (rc == BDD_OK) rc = h->sweep(true, kUpdate, s);
       if (rc == BDD_OK && cudaEventRecord(e[1], s) != cudaSuccess) rc = BDD_ECUDA;
       if (rc == BDD_OK) rc = h->cut(true, s);
@@ -1339,7 +1649,7 @@ int bdd_iterate(bdd_solver *h, int n_iter, double *lower_bound, float *lambda, f
   RC(h->begin(s));
   if (lower_bound && n_iter == 0) {
     CK(cudaMemsetAsync(h->d_iter, 0, sizeof(int), s));
-    RC(h->pending(true, s));
+    RC(h->direct ? h->direct_energy(true, s) : h->pending(true, s));
   }
   const size_t bytes = sizeof(float) * (size_t)h->nnz;
   if (lambda && bytes) CK(cudaMemcpyAsync(lambda, h->d_out_lam, bytes, cudaMemcpyDeviceToHost, s));
@@ -1365,7 +1675,10 @@ int bdd_set_costs(bdd_solver *h, const float *c) {
   RC(h->begin(h->stream));
   ++h->state_gen;
   if (h->n) CK(cudaMemcpyAsync(h->d_c, c, sizeof(float) * h->n, cudaMemcpyHostToDevice, h->stream));
-  h->drop_graphs();  // the bound constant is baked into the captured reductions
+  if (h->direct)
+    RC(h->put_const(h->stream));
+  else
+    h->drop_graphs();  // the bound constant is baked into the captured reductions
   RC(h->restart(h->stream));
   RC(h->end(h->stream));
   CK(cudaStreamSynchronize(h->stream));
@@ -1638,6 +1951,7 @@ int bdd_export_canonical(const bdd_solver *h, int *bdd_row, int *bdd_depth, int 
     std::copy(H.hi.begin(), H.hi.end(), hi);
     return BDD_OK;
   }
+  if (h->direct) return export_direct(h, bdd_row, bdd_depth, occ_var, occ_csr, occ_width, lo, hi);
   // read the slabs back (from the device, or the host copy of the layout) and undo the tiles
   const long long O = h->O, N = h->N, nb = h->nb;
   hvec<int> off(O + 1), var(O), depth(nb), lohi(2 * N);
@@ -1735,11 +2049,15 @@ int bdd_get_state(const bdd_solver *h_in, float *lambda, float *pending) {
   if (lambda) {
     RC(h->ensure_outputs());
     if (h->nnz) CK(cudaMemsetAsync(h->d_out_lam, 0, sizeof(float) * h->nnz, s));
-    if (h->O && scatter_lambda_launch(h->d_lam, h->d_share_occ, h->d_occ_csr, h->d_out_lam, (int)h->O, false,
-                                      s))
+    if (h->direct) {
+      if (direct_scatter_launch(h->direct_params(true), h->Od, h->d_out_lam, false, s)) return BDD_ECUDA;
+    } else if (h->O && scatter_lambda_launch(h->d_lam, h->d_share_occ, h->d_occ_csr, h->d_out_lam, (int)h->O, false,
+                                             s)) {
       return BDD_ECUDA;
+    }
     if (h->nnz) CK(cudaMemcpyAsync(lambda, h->d_out_lam, sizeof(float) * h->nnz, cudaMemcpyDeviceToHost, s));
   }
+  if (pending && h->direct) RC(h->direct_pending(s));
   if (pending && h->n) CK(cudaMemcpyAsync(pending, h->d_P, sizeof(float) * h->n, cudaMemcpyDeviceToHost, s));
   RC(h->end(s));
   CK(cudaStreamSynchronize(s));
@@ -1756,6 +2074,20 @@ int bdd_set_state(bdd_solver *h, const float *lambda, const float *pending) {
   RC(h->begin(s));
   ++h->state_gen;
   if (h->nnz) CK(cudaMemcpyAsync(h->d_out_lam, lambda, sizeof(float) * h->nnz, cudaMemcpyHostToDevice, s));
+  if (h->direct) {
+    if (direct_gather_launch(h->d_out_lam, h->d_occ_csr, h->d_lam, h->Od, s)) return BDD_ECUDA;
+    if (h->n && pending)
+      CK(cudaMemcpyAsync(h->d_P, pending, sizeof(float) * h->n, cudaMemcpyHostToDevice, s));
+    // differences that sum to P: P_i at i's first occurrence, 0 at the others
+    CK(cudaMemsetAsync(h->d_diff_b, 0, sizeof(float) * (size_t)std::max<long long>(h->Od + h->ext, 1), s));
+    if (pending && direct_set_pending_launch(h->d_home, h->d_var_ptr, h->d_P, h->Od, h->d_diff_b, h->n, s))
+      return BDD_ECUDA;
+    RC(h->direct_heavy(false, s));
+    RC(h->direct_energy(false, s));
+    RC(h->end(s));
+    CK(cudaStreamSynchronize(s));
+    return BDD_OK;
+  }
   if (h->O && gather_lambda_launch(h->d_out_lam, h->d_occ_csr, h->d_lam, (int)h->O, s)) return BDD_ECUDA;
   if (h->n) {
     if (pending)
@@ -1793,6 +2125,7 @@ int bdd_bound_parts(bdd_solver *h, int nparts, const long long *row_off, const l
   CK(cudaMemcpyAsync(h->d_part_off, row_off, sizeof(long long) * (nparts + 1), cudaMemcpyHostToDevice, s));
   CK(cudaMemcpyAsync(h->d_part_off + nparts + 1, var_off, sizeof(long long) * (nparts + 1), cudaMemcpyHostToDevice,
                      s));
+  if (h->direct) RC(h->direct_pending(s));
   if (part_bounds_launch(h->d_bdd_E, h->d_bdd_row, (int)h->nb, h->d_E_row, h->m, h->d_part_off,
                          h->d_part_off + nparts + 1, nparts, h->d_var_ptr, h->d_P, h->d_c, h->d_part_out, s))
     return BDD_ECUDA;

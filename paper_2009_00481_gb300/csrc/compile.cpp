@@ -677,6 +677,203 @@ int build_layout(const HostBDDs &H, Layout *L, bool lanes2, const int *class_of_
   return BDD_OK;
 }
 
+int build_direct_layout(const HostBDDs &H, DirectLayout *L, const int *var_deg) {
+  const long long nb = H.nb(), O = H.O();
+  const int n = H.n;
+  std::atomic<bool> fits{true};
+  parallel_for(nb, 4096, [&](long long b0, long long b1) {
+    for (long long b = b0; b < b1; ++b) {
+      int w = 0;
+      for (long long o = H.bdd_occ0[b]; o < H.bdd_occ0[b + 1]; ++o) w = std::max(w, H.occ_width[o]);
+      if (w > 2 || H.bdd_depth[b] > kLaneDeepDepth) fits.store(false);
+    }
+  });
+  if (!fits.load()) return BDD_ETOOBIG;
+  // stable counting sort by depth, deepest first; ties keep ascending row order
+  const int D = H.max_depth;
+  std::vector<long long> cnt(D + 2, 0);
+  for (long long b = 0; b < nb; ++b) cnt[D - H.bdd_depth[b] + 1]++;
+  for (int t = 0; t <= D; ++t) cnt[t + 1] += cnt[t];
+  L->bdd_perm.resize(nb);
+  for (long long b = 0; b < nb; ++b) L->bdd_perm[cnt[D - H.bdd_depth[b]]++] = (int)b;
+  L->bdd_depth.resize(nb);
+  parallel_for(nb, 1 << 14, [&](long long s0, long long s1) {
+    for (long long t = s0; t < s1; ++t) L->bdd_depth[t] = H.bdd_depth[L->bdd_perm[t]];
+  });
+  // tiles of at most 32 BDDs, each a rectangle of its deepest BDD's depth; a depth that fills a tile
+  // starts one of its own (a tile of one depth can be a chain tile)
+  std::vector<long long> run(D + 2, 0);  // BDDs of each depth
+  for (long long s = 0; s < nb; ++s) run[L->bdd_depth[s]]++;
+  long long od = 0;
+  for (long long s = 0; s < nb;) {
+    const int depth = L->bdd_depth[s];
+    long long e = s + 1;
+    while (e < nb && e - s < 32 && (L->bdd_depth[e] == L->bdd_depth[e - 1] || run[L->bdd_depth[e]] < 32)) ++e;
+    const int t[4] = {(int)od, (int)s, (int)(e - s), depth};
+    L->tile.insert(L->tile.end(), t, t + 4);
+    od += 32LL * depth;
+    if (od > INT_MAX) return BDD_ETOOBIG;
+    s = e;
+  }
+  const long long nt = (long long)L->tile.size() / 4;
+  L->n_tiles = (int)nt;
+  for (int c = 1; c < kWarpClasses + 2; ++c) L->class_tile_off[c] = (int)nt;
+  L->Od = od;
+  L->code.resize(od);
+  L->ref.resize(od);
+  L->csr.resize(od);
+  L->var.resize(od);
+  L->occ_of_canon.resize(O);
+  // (a top arc above a last layer, which no non-skipping BDD has, would not fit the code)
+  std::atomic<bool> bad{false};
+  auto arc = [&](int x, bool last) -> unsigned {
+    if ((x >= 0) == last && x != kBot) bad.store(true);
+    return x >= 0 ? (unsigned)x : x == kTop ? 0u : kDirectBot;
+  };
+  std::atomic<int> deep_depth{0};
+  std::atomic<bool> all_chains{true};
+  parallel_for(nt, 64, [&](long long t0, long long t1) {
+    for (long long t = t0; t < t1; ++t) {
+      const long long o0 = L->tile[4 * t];
+      const int b0 = L->tile[4 * t + 1], cb_n = L->tile[4 * t + 2], depth = L->tile[4 * t + 3];
+      bool deep = depth > kLaneRegDepth;
+      bool chain = L->bdd_depth[b0 + cb_n - 1] == depth;
+      unsigned mask = 0;
+      for (int q = 0; q < 32; ++q) {
+        const int cb = q < cb_n ? L->bdd_perm[b0 + q] : -1;
+        const int d = cb >= 0 ? H.bdd_depth[cb] : 0;
+        for (int l = 0; l < depth; ++l) {
+          const long long o = o0 + 32LL * l + q;
+          if (l >= d) {  // padding: no arcs, its own place for its difference
+            L->code[o] = kDirectPad;
+            L->ref[o] = (int)o;
+            L->csr[o] = -1;
+            L->var[o] = -1;
+            continue;
+          }
+          const long long co = H.bdd_occ0[cb] + l, cn = H.occ_node0[co];
+          const bool last = l + 1 == d;
+          unsigned code = arc(H.lo[cn], last) | arc(H.hi[cn], last) << 2;
+          if (H.occ_width[co] == 2) {
+            const unsigned c1 = arc(H.lo[cn + 1], last) | arc(H.hi[cn + 1], last) << 2;
+            if (c1 == (kDirectNoNode1 >> 4)) bad.store(true);  // a node without a path to top
+            code |= c1 << 4;
+          } else {
+            code |= kDirectNoNode1;
+          }
+          L->code[o] = (unsigned char)code;
+          L->csr[o] = H.occ_csr[co];
+          L->var[o] = H.occ_var[co];
+          L->occ_of_canon[co] = (int)o;
+          deep |= var_deg[H.occ_var[co]] > 8;
+          if (l < kLaneRegDepth && var_deg[H.occ_var[co]] > 2) mask |= 1u << l;
+          if (l > 0 && !last && code != kDirectChain) chain = false;
+        }
+      }
+      L->tile[4 * t + 3] |= (int)(mask << kTileMaskShift) | (chain ? kTileChain : 0);
+      if (!chain || deep) all_chains.store(false);
+      if (deep) {
+        L->tile[4 * t + 2] |= kTileDeep;
+        int seen = deep_depth.load();
+        while (seen < depth && !deep_depth.compare_exchange_weak(seen, depth)) {
+        }
+      }
+    }
+  });
+  if (bad.load()) return BDD_EINVAL;
+  L->deep_depth = deep_depth.load();
+  L->chains = all_chains.load();
+  // occurrences of every variable in ascending row order (canonical occurrence order)
+  std::vector<long long> ptr(n + 1);
+  parallel_prefix(var_deg, (long long)n, ptr.data(), (int *)nullptr);
+  L->var_ptr.resize(n + 1);
+  std::vector<int> fill(n + 1, 0);
+  parallel_for(n + 1, 1 << 16, [&](long long a, long long e) {
+    for (long long i = a; i < e; ++i) L->var_ptr[i] = (int)ptr[i];
+  });
+  hvec<int> list(O);
+  parallel_for(O, 1 << 16, [&](long long a, long long e) {
+    for (long long co = a; co < e; ++co) {
+      const int i = H.occ_var[co];
+      list[ptr[i] + __atomic_fetch_add(&fill[i], 1, __ATOMIC_RELAXED)] = (int)co;
+    }
+  });
+  // groups of the grouped values by capacity (4, 8, 16, 32, heavy): a region each, its variables
+  // in index order; ranks from counts per chunk of variables
+  constexpr int kRegions = 5;
+  auto region = [](int d) { return d <= 4 ? 0 : d <= 8 ? 1 : d <= 16 ? 2 : d <= kGatherMax ? 3 : 4; };
+  constexpr long long kChunk = 1 << 16;
+  const long long nch = (n + kChunk - 1) / kChunk;
+  std::vector<long long> size_at(kRegions * (nch + 1), 0), heavy_at(nch + 1, 0);
+  auto room = [&](int r, int d) { return r < 4 ? (4LL << r) : (d + 3LL) / 4 * 4; };
+  parallel_for(nch, 1, [&](long long c0, long long c1) {
+    for (long long c = c0; c < c1; ++c)
+      for (long long i = c * kChunk; i < std::min<long long>(n, (c + 1) * kChunk); ++i)
+        if (var_deg[i] > 2) {
+          const int r = region(var_deg[i]);
+          size_at[kRegions * (c + 1) + r] += room(r, var_deg[i]);
+          heavy_at[c + 1] += r == 4;
+        }
+  });
+  long long start[kRegions + 1] = {0};
+  for (long long c = 0; c < nch; ++c) {
+    for (int r = 0; r < kRegions; ++r) size_at[kRegions * (c + 1) + r] += size_at[kRegions * c + r];
+    heavy_at[c + 1] += heavy_at[c];
+  }
+  for (int r = 0; r < kRegions; ++r)
+    start[r + 1] = (start[r] + (nch ? size_at[kRegions * nch + r] : 0) + 31) / 32 * 32;
+  L->heavy0 = start[4];
+  L->ext = start[kRegions];
+  if (L->ext > (long long)kRefPlace || od + L->ext > INT_MAX) return BDD_ETOOBIG;
+  L->ext_deg.resize(L->ext / 4);
+  std::fill(L->ext_deg.begin(), L->ext_deg.end(), (unsigned char)0);
+  L->heavy.resize(4 * (nch ? heavy_at[nch] : 0));
+  L->heavy_of.resize(L->ext - L->heavy0);
+  std::fill(L->heavy_of.begin(), L->heavy_of.end(), 0);
+  L->home.resize(n);
+  parallel_for(nch, 1, [&](long long c0, long long c1) {
+    for (long long c = c0; c < c1; ++c) {
+      long long at[kRegions], hv = heavy_at[c];
+      for (int r = 0; r < kRegions; ++r) at[r] = start[r] + size_at[kRegions * c + r];
+      for (long long i = c * kChunk; i < std::min<long long>(n, (c + 1) * kChunk); ++i) {
+        const int d = var_deg[i];
+        int *s = list.data() + ptr[i];
+        L->home[i] = 0;
+        if (d == 0) continue;
+        if (d <= kGatherMax) {  // insertion sort of a short list
+          for (int x = 1; x < d; ++x)
+            for (int y = x; y > 0 && s[y - 1] > s[y]; --y) std::swap(s[y - 1], s[y]);
+        } else {
+          std::sort(s, s + d);
+        }
+        if (d <= 2) {
+          const int o1 = L->occ_of_canon[s[0]], o2 = L->occ_of_canon[s[d - 1]];
+          L->ref[o1] = o2;
+          L->ref[o2] = o1;
+          L->home[i] = o1;
+          continue;
+        }
+        const int r = region(d);
+        const long long base = at[r];
+        at[r] += room(r, d);
+        const unsigned k = d <= 8 ? d - 3 : d <= 16 ? kRefMid : kRefLong;
+        const unsigned tag = 0x80000000u | k << kRefShift;
+        for (int x = 0; x < d; ++x) L->ref[L->occ_of_canon[s[x]]] = (int)(tag | (unsigned)(base + x));
+        L->home[i] = (int)(tag | (unsigned)base);
+        if (r < 4) {
+          for (long long g = base / 4; g < (base + room(r, d)) / 4; ++g) L->ext_deg[g] = (unsigned char)d;
+        } else {
+          const int h[4] = {(int)i, (int)base, d, 0};
+          std::copy(h, h + 4, L->heavy.begin() + 4 * hv);
+          for (int x = 0; x < d; ++x) L->heavy_of[base - L->heavy0 + x] = (int)hv;
+          ++hv;
+        }
+      }
+    }
+  });
+  return BDD_OK;
+}
+
 std::vector<int> balanced_cuts(const HostBDDs &H, const int *rank, int k) {
   std::vector<int> cuts;
   const int n = H.n;

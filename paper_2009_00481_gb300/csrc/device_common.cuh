@@ -75,4 +75,75 @@ __device__ __forceinline__ float team_sum(float v) {
   return __shfl_sync(kFull, v, (threadIdx.x & 31) & ~(T - 1));
 }
 
+// wait for the kernel this launch depends on (programmatic dependent launch); a no-op without one
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// mbarrier and bulk-copy (TMA) primitives.  A window's copies complete on its buffer's
+// mbarrier: one lane posts the expected byte count and issues the copies; every lane waits for
+// the phase with a bounded poll.
+__device__ __forceinline__ unsigned smem_u32(const void *ptr) { return (unsigned)__cvta_generic_to_shared(ptr); }
+__device__ __forceinline__ void bar_init(unsigned long long *bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void bar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
+__device__ __forceinline__ void bar_expect(unsigned long long *bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool bar_try_wait(unsigned long long *bar, unsigned parity) {
+  unsigned ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// the GPU's global nanosecond timer
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+// bounded wait for phase `parity`; false if it did not complete within `ns` nanoseconds
+__device__ __forceinline__ bool bar_wait_ns(unsigned long long *bar, unsigned parity, unsigned long long ns) {
+  if (bar_try_wait(bar, parity)) return true;
+  const unsigned long long t0 = global_ns();
+  while (!bar_try_wait(bar, parity))
+    if (global_ns() - t0 > ns) return false;
+  return true;
+}
+// Time limit of a wait on a window's bulk copies.  Copies that were issued always complete, in
+// microseconds, so this limit only guards against a fault elsewhere; it is independent of
+// bdd_options.spin_limit (the grid-barrier poll limit).
+constexpr unsigned long long kRingWaitNs = 2000000000ull;
+__device__ __forceinline__ void bulk_copy(void *dst, const void *src, unsigned bytes, unsigned long long *bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+// generic-proxy writes to global memory (earlier phases of a persistent launch) before bulk reads
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+// generic-proxy writes to this block's shared memory before bulk copies (async proxy) into it
+__device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Asynchronous global -> shared copies (cp.async): a warp issues all copies of a stage back to
+// back and waits once, instead of one load round trip per element.  Data written by other
+// blocks of a persistent launch is read only after a grid barrier, whose fences order those
+// writes before these reads.
+__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// wait until at most N of this thread's committed groups are still in flight
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 }  // namespace bdd

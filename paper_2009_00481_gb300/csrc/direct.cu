@@ -1,0 +1,794 @@
+// Sweeps of the direct plan (see DirectLayout in internal.h): plain min-sum solvers whose sweeps form
+// the pending shares themselves, so that an iteration is two kernels and nothing between them.
+//
+// Lane tiles: one lane per BDD of width <= 2, 32 BDDs per warp.  A warp loads its tile's
+// multipliers, lane codes and differences at once (a rectangle: the addresses follow from the
+// tile's first occurrence), recomputes the messages of the other direction from the multipliers,
+// and walks the layers with everything in registers (up to kLaneRegDepth layers, no variable in more
+// than eight rows) or shared memory.
+// The messages therefore never go through memory: they are functions of the multipliers the
+// sweep before left behind, evaluated with that sweep's own operations, so they are its bits.
+//
+// What bounds the sweeps: on a batch of 32 Potts grids (30.9 M occurrences) a forward sweep moves 0.65 GB
+// in 148 us (4.4 TB/s, two thirds of the copy rate; a backward one 138 us), where the windowed lane
+// tiles moved 1.13 GB in 232 us and two pending passes followed in 98 and 121 us; the rest is load
+// latency at 24 warps per SM.  On small instances (20x20x3 Potts, 156 tiles) a sweep is one dependent
+// chain -- refs, differences, the walk -- of about 2 us, and an iteration 5.8 us against 11.0 us with
+// four kernels.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "device_common.cuh"
+#include "internal.h"
+
+namespace bdd {
+namespace {
+
+// ---------------------------------------------------------------------------------------
+// pending shares from the recorded differences
+// ---------------------------------------------------------------------------------------
+// pending sum and share of an occurrence of a variable in three or more rows (r < 0)
+struct Share {
+  float P, share;
+};
+
+// the first eight values of a group of at most eight (zeros otherwise), issued ahead of their use
+struct Group {
+  float4 a, b;
+};
+__device__ __forceinline__ Group load_group(const DirectParams &p, int r) {
+  Group g;
+  g.a = g.b = make_float4(0.f, 0.f, 0.f, 0.f);
+  const unsigned k = ((unsigned)r >> kRefShift) & 7u, place = (unsigned)r & kRefPlace;
+  if (r < 0 && k < kRefMid) {
+    const unsigned base = place & ~(k < 2u ? 3u : 7u);
+    g.a = *reinterpret_cast<const float4 *>(p.ein + base);
+    if (k >= 2u) g.b = *reinterpret_cast<const float4 *>(p.ein + base + 4);
+  }
+  return g;
+}
+
+// a variable in more than eight rows
+__device__ __forceinline__ Share long_share(const DirectParams &p, unsigned k, unsigned place) {
+  const int deg = p.ext_deg[place >> 2];
+  if (deg == 0) {
+    const float2 h = p.heavy[p.heavy_of[place - p.heavy0]];
+    return {h.x, h.y};
+  }
+  const unsigned cap = k == kRefMid ? 16u : 32u;
+  const float *v = p.ein + (place & ~(cap - 1u));
+  float P = 0.f;
+  for (unsigned j = 0; j < cap; j += 16) {  // unused values are 0
+    float4 q[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) q[x] = *reinterpret_cast<const float4 *>(v + j + 4 * x);
+#pragma unroll
+    for (int x = 0; x < 4; ++x) P = P + q[x].x + q[x].y + q[x].z + q[x].w;
+  }
+  return {P, P / (float)deg};
+}
+
+// the additions of the pending pass: from 0, in ascending row order (unused values are 0, and a sum
+// that starts from 0 is never -0, so they change nothing)
+__device__ __forceinline__ Share group_share(int r, const Group &g) {
+  const unsigned k = ((unsigned)r >> kRefShift) & 7u;
+  float P = 0.f + g.a.x + g.a.y + g.a.z + g.a.w;
+  if (k >= 2u) P = P + g.b.x + g.b.y + g.b.z + g.b.w;
+  return {P, P / (float)(3u + k)};
+}
+
+__device__ __forceinline__ bool is_long(int r) { return r < 0 && (((unsigned)r >> kRefShift) & 7u) >= kRefMid; }
+
+// whether this occurrence is the one that adds its variable's slack to the bound
+__device__ __forceinline__ bool adds_slack(int r, int o) {
+  if (r >= 0) return r >= o;
+  const unsigned k = ((unsigned)r >> kRefShift) & 7u;
+  return k < kRefMid && ((unsigned)r & (k < 2u ? 3u : 7u)) == 0u;
+}
+__device__ __forceinline__ bool long_adds_slack(const DirectParams &p, int r) {
+  const unsigned k = ((unsigned)r >> kRefShift) & 7u, place = (unsigned)r & kRefPlace;
+  if (k == kRefMid) return (place & 15u) == 0u;
+  if (p.ext_deg[place >> 2]) return (place & 31u) == 0u;
+  return place == (unsigned)p.heavy0 || p.heavy_of[place - p.heavy0] != p.heavy_of[place - p.heavy0 - 1];
+}
+
+// a variable in one row (r == o) or two
+__device__ __forceinline__ Share near_share(int r, int o, float own, float mate) {
+  if (r == o) return {0.f + own, 0.f + own};
+  const float P = own + mate;  // 0 + a + b in either order
+  return {P, 0.5f * P};
+}
+
+// A lane's share of the bound: Knuth's TwoSum in FP32 with the rounding errors in lo; after every
+// tile the pair is renormalised (lo below half an ulp of hi), so the sum keeps about 47 bits over
+// any number of tiles.  One FP64 addition per tile instead cost 16 cycles of an SM each (this part's
+// FP64 rate is 1/64 of its FP32 rate): 30 us of a 200 us sweep.
+struct BoundPair {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = hi + x, xv = t - hi;
+    lo += (hi - (t - xv)) + (x - xv);
+    hi = t;
+  }
+  __device__ __forceinline__ void renormalise() {
+    if (!(fabsf(lo) < inf())) lo = 0.f;  // an infinite or NaN term: hi alone is the plain sum's value
+    const float t = hi + lo;
+    lo = lo - (t - hi);
+    hi = t;
+  }
+  __device__ __forceinline__ double value() const { return fabsf(lo) < inf() ? (double)hi + (double)lo : (double)hi; }
+};
+
+__device__ __forceinline__ float mm_step(float m0, float m1) {
+  // a +inf min-marginal (a row forcing x_i) transfers nothing
+  return (m0 < inf() && m1 < inf()) ? m1 - m0 : 0.f;
+}
+
+// ---------------------------------------------------------------------------------------
+// lane codes
+// ---------------------------------------------------------------------------------------
+// Every function takes the code in byte `at` of a word.  Message of the arc at bits k, k + 1: node 0
+// (a last layer's arc to top, too: the walk starts from messages 0 and +inf behind it) or 1 of the
+// next layer, or bot
+__device__ __forceinline__ float pull(unsigned c, int k, float x0, float x1) {
+  const float node = c & (1u << k) ? x1 : x0;
+  return c & (2u << k) ? inf() : node;
+}
+// the path cost v along that arc relaxes the node it leads to
+__device__ __forceinline__ void push(unsigned c, int k, float v, float &n0, float &n1) {
+  const bool one = c & (1u << k);
+  const float live = c & (2u << k) ? inf() : v;
+  n0 = fminf(n0, one ? inf() : live);
+  n1 = fminf(n1, one ? live : inf());
+}
+__device__ __forceinline__ void step_back(unsigned c, int at, float lam, float &x0, float &x1) {
+  const int k = 8 * at;
+  const float n0 = fminf(pull(c, k, x0, x1), lam + pull(c, k + 2, x0, x1));
+  const float n1 = fminf(pull(c, k + 4, x0, x1), lam + pull(c, k + 6, x0, x1));
+  x0 = n0;
+  x1 = n1;
+}
+__device__ __forceinline__ void step_on(unsigned c, int at, float lam, float &f0, float &f1) {
+  const int k = 8 * at;
+  float n0 = inf(), n1 = inf();
+  push(c, k, f0, n0, n1);
+  push(c, k + 2, f0 + lam, n0, n1);
+  push(c, k + 4, f1, n0, n1);
+  push(c, k + 6, f1 + lam, n0, n1);
+  f0 = n0;
+  f1 = n1;
+}
+// min-marginals of a layer: forward messages f, messages x of the next layer's nodes
+__device__ __forceinline__ float2 layer_mm(unsigned c, int at, float lam, float f0, float f1, float x0, float x1) {
+  const int k = 8 * at;
+  return make_float2(fminf(f0 + pull(c, k, x0, x1), f1 + pull(c, k + 4, x0, x1)),
+                     fminf(f0 + lam + pull(c, k + 2, x0, x1), f1 + lam + pull(c, k + 6, x0, x1)));
+}
+
+// (Decoding the arcs is most of a walk's work: a forward sweep of 13.6 M occurrences took 48 M warp
+// instructions with it and takes 32 M where the layers are chain layers.)
+// A chain layer: node 0's arcs to nodes 0 and 1, node 1's 0-arc to node 1 and its 1-arc to bot -- every
+// inner layer of a row "exactly / at most one of" and of a flow row.  The same results (the terms
+// left out are +inf) without decoding an arc.
+__device__ __forceinline__ void chain_back(float lam, float &x0, float x1) { x0 = fminf(x0, lam + x1); }
+__device__ __forceinline__ void chain_on(float lam, float f0, float &f1) { f1 = fminf(f0 + lam, f1); }
+__device__ __forceinline__ float2 chain_mm(float lam, float f0, float f1, float x0, float x1) {
+  return make_float2(fminf(f0 + x0, f1 + x1), f0 + lam + x1);
+}
+
+__device__ __forceinline__ void store_diff(const DirectParams &p, int r, int o, float d) {
+  // (the grouped values lie behind the occurrences)
+  p.dout[BDD_IN(p, r >= 0 ? o : (int)((unsigned)r & kRefPlace) + (int)p.n_occ, p.n_diff)] = d;
+}
+
+// One lane tile of depth D in registers: 21 bytes per occurrence and sweep (code 1, ref 4, multiplier
+// 4 + 4, differences 4 + 4; the mates mostly lie in the same tile).  CHAIN: every BDD of the tile has
+// depth D and chain layers between its first and its last (kTileChain); their codes are not read.
+template <int D, bool FWD, int MODE, bool CHAIN>
+__device__ __forceinline__ void lane_tile(const DirectParams &p, const int4 &t, int kind, BoundPair &sum) {
+  const int lane = threadIdx.x & 31;
+  const int o = (int)BDD_IN(p, t.x + lane, p.n_occ - 32 * (D - 1));
+  constexpr int W = (D + 3) / 4;
+  auto inner = [](int l) { return CHAIN && l > 0 && l < D - 1; };
+  const unsigned grouped = (unsigned)kind >> kTileMaskShift;  // layers with grouped values on any lane
+  unsigned code[W];  // four layers' codes a word
+  int ref[D];
+#pragma unroll
+  for (int w = 0; w < W; ++w) code[w] = 0u;
+#pragma unroll
+  for (int l = 0; l < D; ++l)
+    if (!inner(l)) code[l / 4] |= (unsigned)p.code[o + 32 * l] << (8 * (l % 4));
+#pragma unroll
+  for (int l = 0; l < D; ++l) ref[l] = p.ref[o + 32 * l];
+  pdl_wait();
+  // (multipliers and own differences go out with the refs, whose arrival only the mates wait for)
+  float lam[D], own[D], mate[D];
+#pragma unroll
+  for (int l = 0; l < D; ++l) lam[l] = p.lam[o + 32 * l];
+#pragma unroll
+  for (int l = 0; l < D; ++l) own[l] = p.din[o + 32 * l];
+#pragma unroll
+  for (int l = 0; l < D; ++l) mate[l] = p.din[ref[l] >= 0 ? BDD_IN(p, ref[l], p.n_diff) : o + 32 * l];
+  // the first layer's group is under way while the messages are recomputed (a Potts edge row has
+  // its only variable in more than two rows there)
+  Group g0{};
+  if (grouped & 1u) g0 = load_group(p, ref[0]);
+
+  auto back = [&](int l, float la, float &y0, float &y1) {
+    if (inner(l)) chain_back(la, y0, y1);
+    else step_back(code[l / 4], l % 4, la, y0, y1);
+  };
+  auto on = [&](int l, float la, float &f0, float &f1) {
+    if (inner(l)) chain_on(la, f0, f1);
+    else step_on(code[l / 4], l % 4, la, f0, f1);
+  };
+  auto mm = [&](int l, float la, float f0, float f1, float y0, float y1) {
+    return inner(l) ? chain_mm(la, f0, f1, y0, y1) : layer_mm(code[l / 4], l % 4, la, f0, f1, y0, y1);
+  };
+  float x0[D], x1[D];  // messages of the other direction: of the next layer (FWD), of this one
+  float e = 0.f;
+  auto messages = [&](const float (&cost)[D]) {
+    if (FWD) {
+      float y0 = 0.f, y1 = inf();
+#pragma unroll
+      for (int l = D - 1; l >= 0; --l) {
+        x0[l] = y0;
+        x1[l] = y1;
+        back(l, cost[l], y0, y1);
+      }
+      e = y0;
+    } else {
+      float f0 = 0.f, f1 = inf();
+#pragma unroll
+      for (int l = 0; l < D; ++l) {
+        x0[l] = f0;
+        x1[l] = f1;
+        if (l + 1 < D) on(l, cost[l], f0, f1);
+      }
+    }
+  };
+  if (MODE != kDirectFolded) messages(lam);
+  const bool bound = FWD && MODE != kDirectFolded && p.sum_bound;
+  float shr[D];
+  auto near = [&](int l) {
+    const Share s = near_share(ref[l], o + 32 * l, own[l], mate[l]);
+    shr[l] = s.share;
+    if (bound) sum.add(ref[l] >= o + 32 * l ? fminf(s.P, 0.f) : 0.f);
+  };
+  auto either = [&](int l, const Group &g) {
+    const Share s = ref[l] < 0 ? group_share(ref[l], g) : near_share(ref[l], o + 32 * l, own[l], mate[l]);
+    shr[l] = s.share;
+    if (bound) sum.add(adds_slack(ref[l], o + 32 * l) ? fminf(s.P, 0.f) : 0.f);
+  };
+  if (grouped & 1u)
+    either(0, g0);
+  else
+    near(0);
+#pragma unroll
+  for (int l = 1; l < D; l += 2) {  // groups two layers at a time
+    constexpr int last = D - 1;
+    const int m = l < last ? l + 1 : last;
+    if ((grouped >> l) & 3u) {  // (no group outlives its layers: it would be carried from tile to tile)
+      const Group ga = load_group(p, ref[l]), gb = load_group(p, ref[m]);
+      either(l, ga);
+      if (l < last) either(m, gb);
+    } else {
+      near(l);
+      if (l < last) near(m);
+    }
+  }
+  // (keeps the compiler from holding the decoded arcs of every layer from one walk to the next)
+#pragma unroll
+  for (int w = 0; w < W; ++w) asm volatile("" : "+r"(code[w]));
+  const bool mine = lane < t.z;  // a BDD, not padding
+  if (FWD && MODE != kDirectFolded) {
+    if (bound) {
+      sum.add(mine ? e : 0.f);
+      sum.renormalise();
+    }
+    if (MODE == kDirectEnergy) {
+      if (mine) p.bdd_E[BDD_IN(p, t.y + lane, p.n_bdd)] = e;
+      return;
+    }
+  }
+  if (MODE == kDirectFolded) {
+#pragma unroll
+    for (int l = 0; l < D; ++l) lam[l] = lam[l] + shr[l];
+    messages(lam);
+    float f0 = 0.f, f1 = inf();
+#pragma unroll
+    for (int l = 0; l < D; ++l) {
+      const float2 m = mm(l, lam[l], f0, f1, x0[l], x1[l]);
+      const long long c = p.csr[o + 32 * l];
+      if (c >= 0) {
+        p.out_m0[BDD_IN(p, c, p.n_csr)] = m.x;
+        p.out_m1[BDD_IN(p, c, p.n_csr)] = m.y;
+      }
+      on(l, lam[l], f0, f1);
+    }
+    return;
+  }
+  // eqs. arc-marginal / marginal-aggregation, the damped eq. mma-update step, Alg. 2 / Alg. 3
+  float y0 = 0.f, y1 = inf();
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    const int l = FWD ? j : D - 1 - j;
+    float la = lam[l] + shr[l];
+    const float2 m = FWD ? mm(l, la, y0, y1, x0[l], x1[l]) : mm(l, la, x0[l], x1[l], y0, y1);
+    const float dd = p.omega * mm_step(m.x, m.y);
+    la -= dd;
+    p.lam[o + 32 * l] = la;
+    store_diff(p, ref[l], o + 32 * l, dd);
+    if (FWD)
+      on(l, la, y0, y1);
+    else
+      back(l, la, y0, y1);
+  }
+  if (!FWD && mine) p.bdd_E[BDD_IN(p, t.y + lane, p.n_bdd)] = y0;
+}
+
+// The columns of a deep lane tile in shared memory (one per lane).
+struct DeepColumns {
+  float2 *xs;
+  float *lams, *shrs;
+  int *refs;
+  unsigned char *codes;
+};
+__device__ __forceinline__ DeepColumns deep_columns(char *smem, int depth) {
+  const int lane = threadIdx.x & 31;
+  DeepColumns c;
+  c.xs = reinterpret_cast<float2 *>(smem) + lane;
+  c.lams = reinterpret_cast<float *>(smem + 32 * 8 * (size_t)depth) + lane;
+  c.shrs = c.lams + 32 * depth;
+  c.refs = reinterpret_cast<int *>(c.shrs + 32 * depth);
+  c.codes = reinterpret_cast<unsigned char *>(c.refs - lane + 32 * depth) + lane;
+  return c;
+}
+
+// the values of an occurrence's group (zeros where it has none) and its rows if it is long
+struct WideGroup {
+  float4 v[kGatherMax / 4];
+  int deg;
+};
+__device__ __forceinline__ WideGroup load_wide(const DirectParams &p, int r) {
+  WideGroup g;
+  const unsigned k = ((unsigned)r >> kRefShift) & 7u, place = (unsigned)r & kRefPlace;
+  const int cap = r >= 0 ? 0 : ref_capacity((int)k);
+  g.deg = r < 0 && k >= kRefMid ? p.ext_deg[place >> 2] : -1;
+  const float *v = p.ein + (place & ~(unsigned)(cap - 1));
+  const bool heavy = cap == 32 && place >= (unsigned)p.heavy0;
+#pragma unroll
+  for (int x = 0; x < kGatherMax / 4; ++x) {
+    g.v[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (cap > 4 * x && !heavy) g.v[x] = *reinterpret_cast<const float4 *>(v + 4 * x);
+  }
+  return g;
+}
+__device__ __forceinline__ Share wide_share(const DirectParams &p, int r, const WideGroup &g) {
+  const unsigned k = ((unsigned)r >> kRefShift) & 7u, place = (unsigned)r & kRefPlace;
+  if (g.deg == 0) {
+    const float2 h = p.heavy[p.heavy_of[place - p.heavy0]];
+    return {h.x, h.y};
+  }
+  float P = 0.f;
+#pragma unroll
+  for (int x = 0; x < kGatherMax / 4; ++x) P = P + g.v[x].x + g.v[x].y + g.v[x].z + g.v[x].w;  // unused values are 0
+  return {P, P / (float)(k < kRefMid ? 3 + (int)k : g.deg)};
+}
+
+// Loads of layers l0, l0 + step, ... of a deep tile into its columns: codes, then (after the wait for
+// the sweep before) multipliers and shares, two layers' groups to a round of loads.
+template <bool FWD, int MODE>
+__device__ __forceinline__ void deep_load(const DirectParams &p, const int4 &t, const DeepColumns &c, int l0, int step,
+                                          BoundPair &sum) {
+  const int lane = threadIdx.x & 31, D = t.w;
+  const int o = (int)BDD_IN(p, t.x + lane, p.n_occ - 32 * (D - 1));
+#pragma unroll 4
+  for (int l = l0; l < D; l += step) c.codes[32 * l] = p.code[o + 32 * l];
+  pdl_wait();
+  const bool bound = FWD && MODE != kDirectFolded && p.sum_bound;
+  for (int l = l0; l < D; l += 2 * step) {
+    const int m = l + step < D ? l + step : l;
+    const int ol = o + 32 * l, om = o + 32 * m;
+    const int rl = p.ref[ol], rm = p.ref[om];
+    const float laml = p.lam[ol], lamm = p.lam[om], ownl = p.din[ol], ownm = p.din[om];
+    const float matel = p.din[rl >= 0 ? BDD_IN(p, rl, p.n_diff) : ol], matem = p.din[rm >= 0 ? BDD_IN(p, rm, p.n_diff) : om];
+    const WideGroup gl = load_wide(p, rl), gm = load_wide(p, rm);
+    auto take = [&](int q, int oq, int r, float lam, float own, float mate, const WideGroup &g) {
+      const Share s = r < 0 ? wide_share(p, r, g) : near_share(r, oq, own, mate);
+      if (bound) sum.add((is_long(r) ? long_adds_slack(p, r) : adds_slack(r, oq)) ? fminf(s.P, 0.f) : 0.f);
+      c.lams[32 * q] = MODE == kDirectFolded ? lam + s.share : lam;
+      c.shrs[32 * q] = s.share;
+      c.refs[32 * q] = r;
+    };
+    take(l, ol, rl, laml, ownl, matel, gl);
+    if (m != l) take(m, om, rm, lamm, ownm, matem, gm);
+  }
+  if (bound) sum.renormalise();
+}
+
+// The walks of a deep tile over its columns, by one warp.
+template <bool FWD, int MODE>
+__device__ __forceinline__ void deep_walk(const DirectParams &p, const int4 &t, const DeepColumns &c, bool chain, BoundPair &sum) {
+  const int lane = threadIdx.x & 31, D = t.w;
+  const int o = (int)BDD_IN(p, t.x + lane, p.n_occ - 32 * (D - 1));
+  auto inner = [&](int l) { return chain && l > 0 && l < D - 1; };
+  // messages of the other direction (FWD: of the next layer); a layer's column entries are read a
+  // layer ahead, so the recurrence does not wait on shared memory
+  float y0 = 0.f, y1 = inf();
+  {
+    const int l0 = FWD ? D - 1 : 0, dl = FWD ? -1 : 1;
+    float la = c.lams[32 * l0];
+    unsigned code = c.codes[32 * l0];
+    for (int j = 0; j < D; ++j) {
+      const int l = l0 + j * dl, ln = j + 1 < D ? l + dl : l;
+      const float lan = c.lams[32 * ln];
+      const unsigned coden = c.codes[32 * ln];
+      c.xs[32 * l] = make_float2(y0, y1);
+      if (inner(l)) {
+        if (FWD) chain_back(la, y0, y1);
+        else chain_on(la, y0, y1);
+      } else if (FWD) {
+        step_back(code, 0, la, y0, y1);
+      } else {
+        step_on(code, 0, la, y0, y1);
+      }
+      la = lan;
+      code = coden;
+    }
+  }
+  const bool mine = lane < t.z;
+  if (FWD && MODE != kDirectFolded) {
+    if (p.sum_bound) sum.add(mine ? y0 : 0.f);
+    if (MODE == kDirectEnergy) {
+      if (mine) p.bdd_E[BDD_IN(p, t.y + lane, p.n_bdd)] = y0;
+      return;
+    }
+  }
+  y0 = 0.f;
+  y1 = inf();
+  struct Layer {
+    unsigned code;
+    float2 x;
+    float la, shr;
+    int ref;
+  };
+  auto layer = [&](int l) { return Layer{c.codes[32 * l], c.xs[32 * l], c.lams[32 * l], c.shrs[32 * l], c.refs[32 * l]}; };
+  Layer next = layer(FWD ? 0 : D - 1);
+  for (int j = 0; j < D; ++j) {
+    const int l = FWD ? j : D - 1 - j, ol = o + 32 * l;
+    const Layer q = next;
+    next = layer(j + 1 < D ? (FWD ? l + 1 : l - 1) : l);
+    const unsigned code = q.code;
+    const float2 x = q.x;
+    float la = q.la;
+    if (MODE != kDirectFolded) la += q.shr;  // (folded: added by the load)
+    const float f0 = FWD ? y0 : x.x, f1 = FWD ? y1 : x.y, b0 = FWD ? x.x : y0, b1 = FWD ? x.y : y1;
+    const float2 m = inner(l) ? chain_mm(la, f0, f1, b0, b1) : layer_mm(code, 0, la, f0, f1, b0, b1);
+    if (MODE == kDirectFolded) {
+      const long long at = p.csr[ol];
+      if (at >= 0) {
+        p.out_m0[BDD_IN(p, at, p.n_csr)] = m.x;
+        p.out_m1[BDD_IN(p, at, p.n_csr)] = m.y;
+      }
+    } else {
+      const float dd = p.omega * mm_step(m.x, m.y);
+      la -= dd;
+      p.lam[ol] = la;
+      store_diff(p, q.ref, ol, dd);
+    }
+    if (inner(l)) {
+      if (FWD) chain_on(la, y0, y1);
+      else chain_back(la, y0, y1);
+    } else if (FWD) {
+      step_on(code, 0, la, y0, y1);
+    } else {
+      step_back(code, 0, la, y0, y1);
+    }
+  }
+  if (MODE == kDirectUpdate && !FWD && mine) p.bdd_E[BDD_IN(p, t.y + lane, p.n_bdd)] = y0;
+}
+
+// per-block bound partials into the trace, by one warp in a fixed order
+__device__ __forceinline__ void finish_bound(const double *partial, int nblocks, const DirectParams &p) {
+  const int lane = threadIdx.x & 31;
+  double s = 0.0;
+  for (int k = lane; k < nblocks; k += 32) s += __ldcg(partial + k);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
+  if (lane == 0) {
+    const int it = *p.iter_ctr;
+    if (it < p.trace_cap) p.trace[it] = s + *p.empty_const;
+    *p.iter_ctr = it + 1;
+  }
+}
+
+// Block sum of the lanes' bound terms into the block's partial; in a pass of its own (LAST) the last
+// block to arrive finishes the bound.
+template <int WARPS, bool LAST>
+__device__ __forceinline__ void store_partial(const DirectParams &p, const BoundPair &pair) {
+  double acc = pair.value();
+  __shared__ double red[WARPS];
+  __shared__ bool last;
+  const int warp = threadIdx.x >> 5;
+  pdl_wait();  // (a block without tiles has not waited yet)
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(kFull, acc, off);
+  if ((threadIdx.x & 31) == 0) red[warp] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < WARPS; ++w) s += red[w];
+    p.partial[blockIdx.x] = s;
+    if (LAST) {
+      __threadfence();
+      last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+    }
+  }
+  if (!LAST) return;
+  __syncthreads();
+  if (last && warp == 0) {
+    __threadfence();
+    finish_bound(p.partial, gridDim.x, p);
+    if (threadIdx.x == 0) *p.ticket = 0u;
+  }
+}
+
+// sends for the next tile of this warp (refs, multipliers, differences, codes: a line per lane) while
+// this one is worked on, so that its loads find them in L2
+__device__ __forceinline__ void prefetch_tile(const DirectParams &p, const int4 &t) {
+  const int lane = threadIdx.x & 31, kind = lane / 10, l = lane % 10, D = t.w & kTileDepth;
+  const void *line = kind == 0   ? (const void *)(p.ref + t.x + 32 * l)
+                     : kind == 1 ? (const void *)(p.lam + t.x + 32 * l)
+                     : kind == 2 ? (const void *)(p.din + t.x + 32 * l)
+                                 : (const void *)(p.code + t.x + (l ? 32 * (D - 1) : 0));
+  if (kind == 3 || l < D) asm volatile("prefetch.global.L2 [%0];" ::"l"(line));
+}
+
+// CHAINS: every tile is a chain tile that runs in registers; otherwise the general form.  The chain
+// form needs 80 registers for six blocks per SM (forward / backward sweep of the 32-grid batch: four
+// blocks 193 / 187 us, five 161 / 156, six 150 / 147, seven 146 / 146 with twice the spills, eight
+// 150 / 148); the general one is used where latency counts and takes what it needs.
+template <bool FWD, int MODE, bool CHAINS>
+__global__ void __launch_bounds__(kBlockThreads, CHAINS ? 6 : 3) direct_kernel(const DirectParams p) {
+  extern __shared__ __align__(16) char smem[];
+  if (p.pdl_early) pdl_release();
+  const int warp = threadIdx.x >> 5;
+  if (!FWD && MODE == kDirectUpdate && blockIdx.x == gridDim.x - 1) {  // the block after the tiles'
+    pdl_wait();
+    if (warp == 0 && p.fin_partial) finish_bound(p.fin_partial, p.fin_nblocks, p);
+    return;
+  }
+  const int nblocks = gridDim.x - (!FWD && MODE == kDirectUpdate ? 1 : 0);
+  BoundPair acc;
+  if constexpr (!CHAINS) {  // the deepest tiles, a block each: its warps load the layers, its first walks them
+    if ((int)blockIdx.x < p.n_coop) {
+      int4 t = p.tile[blockIdx.x];
+      const bool chain = t.w & kTileChain;
+      t.z &= kTileDeep - 1;
+      t.w &= kTileDepth;
+      const DeepColumns c = deep_columns(smem, p.deep_depth);
+      deep_load<FWD, MODE>(p, t, c, warp, kWarpsPerBlock, acc);
+      __syncthreads();
+      if (warp == 0) deep_walk<FWD, MODE>(p, t, c, chain, acc);
+    }
+  }
+  const int other = CHAINS ? 0 : p.n_coop;  // tiles and blocks of that kind
+  const int b0 = (int)blockIdx.x - other;
+  const int step = (nblocks - other) * kWarpsPerBlock, k0 = other + b0 * kWarpsPerBlock + warp;
+  auto tile = [&](int k) { return b0 >= 0 && k < p.n_tiles ? p.tile[k] : make_int4(0, 0, 0, 0); };
+  int4 t = tile(k0), t1 = tile(k0 + step);
+  for (int k = k0; t.w; k += step) {
+    const int4 t2 = tile(k + 2 * step);  // (a tile's description arrives a tile before it is asked for)
+    if (t1.w) prefetch_tile(p, t1);
+    const int kind = t.w;
+    const bool chain = t.w & kTileChain;
+    const bool deep = t.z & kTileDeep;
+    t.z &= kTileDeep - 1;
+    t.w &= kTileDepth;
+    if constexpr (!CHAINS) {
+      if (deep) {
+        const DeepColumns c = deep_columns(smem + (size_t)warp * p.warp_depth * kLaneLayerBytes, p.warp_depth);
+        deep_load<FWD, MODE>(p, t, c, 0, 1, acc);
+        deep_walk<FWD, MODE>(p, t, c, chain, acc);
+        t = t1;
+        t1 = t2;
+        continue;
+      }
+    }
+    switch (t.w) {
+#define BDD_LANE_CASE(D)                           \
+  case D:                                          \
+    if (CHAINS || chain)                           \
+      lane_tile<D, FWD, MODE, true>(p, t, kind, acc);    \
+    else                                                 \
+      lane_tile<D, FWD, MODE, false>(p, t, kind, acc);   \
+    break;
+      BDD_LANE_CASE(1)
+      BDD_LANE_CASE(2)
+      BDD_LANE_CASE(3)
+      BDD_LANE_CASE(4)
+      BDD_LANE_CASE(5)
+      BDD_LANE_CASE(6)
+      BDD_LANE_CASE(7)
+      BDD_LANE_CASE(8)
+      BDD_LANE_CASE(9)
+      BDD_LANE_CASE(10)
+#undef BDD_LANE_CASE
+      default:
+        break;
+    }
+    t = t1;
+    t1 = t2;
+  }
+  if (FWD && MODE != kDirectFolded && p.sum_bound) store_partial<kWarpsPerBlock, MODE == kDirectEnergy>(p, acc);
+}
+
+// variables in more than kGatherMax rows: pending sum and share, one warp each (32 values per round
+// of loads, every lane adding them in row order)
+__global__ void __launch_bounds__(kBlockThreads) heavy_kernel(const int4 *heavy, int n_heavy, const float *ein,
+                                                              float2 *out) {
+  const int w = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  int4 h = make_int4(0, 0, 0, 0);
+  if (w < n_heavy) h = heavy[w];
+  pdl_wait();
+  float P = 0.f;
+  for (int k0 = 0; k0 < h.z; k0 += 32) {
+    const float v = k0 + lane < h.z ? ein[h.y + k0 + lane] : 0.f;
+    const int here = min(32, h.z - k0);
+    for (int j = 0; j < here; ++j) P += __shfl_sync(kFull, v, j);
+  }
+  if (w < n_heavy && lane == 0) out[w] = make_float2(P, P / (float)h.z);
+}
+
+// lambda^j_i = c_i / |J_i|, 0 on padding
+__global__ void direct_init_kernel(const int *__restrict__ var, const int *__restrict__ var_ptr,
+                                   const float *__restrict__ c, float *__restrict__ lam, long long Od) {
+  for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < Od; o += (long long)gridDim.x * blockDim.x) {
+    const int i = var[o];
+    lam[o] = i >= 0 ? c[i] / (float)(var_ptr[i + 1] - var_ptr[i]) : 0.f;
+  }
+}
+
+__global__ void direct_pending_kernel(const int *__restrict__ home, const int *__restrict__ ref,
+                                      const int *__restrict__ var_ptr, const float *__restrict__ d, long long ext0,
+                                      float *__restrict__ P, int n) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int deg = var_ptr[i + 1] - var_ptr[i], h = home[i];
+    float s = 0.f;
+    if (deg == 1) {
+      s += d[h];
+    } else if (deg == 2) {
+      s += d[h];
+      s += d[ref[h]];
+    } else if (deg > 2) {
+      const float *v = d + ext0 + ((unsigned)h & kRefPlace);
+      for (int k = 0; k < deg; ++k) s += v[k];
+    }
+    P[i] = s;
+  }
+}
+
+// P_i where i's first difference lies (the others are 0 already)
+__global__ void direct_set_pending_kernel(const int *__restrict__ home, const int *__restrict__ var_ptr,
+                                          const float *__restrict__ P, long long ext0, float *__restrict__ d, int n) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    if (var_ptr[i + 1] == var_ptr[i]) continue;
+    const int h = home[i];
+    d[h >= 0 ? h : ext0 + ((unsigned)h & kRefPlace)] = P[i];
+  }
+}
+
+__global__ void direct_scatter_kernel(const DirectParams p, long long Od, float *__restrict__ out, bool fold) {
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < Od; k += (long long)gridDim.x * blockDim.x) {
+    const long long c = p.csr[k];
+    if (c < 0) continue;
+    float v = p.lam[k];
+    if (fold) {
+      const int o = (int)k, r = p.ref[o];
+      v += is_long(r) ? long_share(p, ((unsigned)r >> kRefShift) & 7u, (unsigned)r & kRefPlace).share
+           : r < 0    ? group_share(r, load_group(p, r)).share
+                      : near_share(r, o, p.din[o], p.din[r]).share;
+    }
+    out[c] = v;
+  }
+}
+
+__global__ void direct_gather_kernel(const float *__restrict__ in, const long long *__restrict__ csr,
+                                     float *__restrict__ lam, long long Od) {
+  for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < Od; o += (long long)gridDim.x * blockDim.x)
+    lam[o] = csr[o] >= 0 ? in[csr[o]] : 0.f;
+}
+
+int status() { return cudaGetLastError() == cudaSuccess ? 0 : -5; }
+int grid_for(long long work) { return (int)std::max<long long>(1, std::min<long long>((work + 255) / 256, 152 * 16)); }
+
+template <typename... Args>
+int launch_pdl(void (*kernel)(Args...), int grid, int block, size_t smem, cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? 0 : -5;
+}
+
+template <bool CHAINS>
+int launch(bool forward, int mode, const DirectParams &p, int grid, size_t smem, cudaStream_t s) {
+  if (mode == kDirectFolded) return launch_pdl(direct_kernel<true, kDirectFolded, CHAINS>, grid, kBlockThreads, smem, s, p);
+  if (mode == kDirectEnergy) return launch_pdl(direct_kernel<true, kDirectEnergy, CHAINS>, grid, kBlockThreads, smem, s, p);
+  if (forward) return launch_pdl(direct_kernel<true, kDirectUpdate, CHAINS>, grid, kBlockThreads, smem, s, p);
+  return launch_pdl(direct_kernel<false, kDirectUpdate, CHAINS>, grid + 1, kBlockThreads, smem, s, p);
+}
+
+}  // namespace
+
+int direct_launch(bool forward, int mode, const DirectParams &p, int grid, size_t smem, cudaStream_t stream) {
+  const int rc = p.chains ? launch<true>(forward, mode, p, grid, smem, stream)
+                          : launch<false>(forward, mode, p, grid, smem, stream);
+  return rc ? rc : status();
+}
+
+int direct_resident_blocks(bool chains, size_t smem, int *blocks) {
+  const cudaError_t e =
+      chains ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, direct_kernel<true, kDirectUpdate, true>, kBlockThreads, smem)
+             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, direct_kernel<true, kDirectUpdate, false>, kBlockThreads, smem);
+  return e == cudaSuccess ? 0 : -5;
+}
+
+int direct_set_smem(size_t smem) {
+  const void *fns[] = {(const void *)direct_kernel<true, kDirectUpdate, false>,
+                       (const void *)direct_kernel<false, kDirectUpdate, false>,
+                       (const void *)direct_kernel<true, kDirectEnergy, false>,
+                       (const void *)direct_kernel<true, kDirectFolded, false>};
+  for (const void *f : fns)
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -5;
+  return 0;
+}
+
+int heavy_launch(const int4 *heavy, int n_heavy, const float *ein, float2 *out, cudaStream_t stream) {
+  if (n_heavy == 0) return 0;
+  const int rc = launch_pdl(heavy_kernel, (n_heavy + kWarpsPerBlock - 1) / kWarpsPerBlock, kBlockThreads, 0, stream, heavy,
+                            n_heavy, ein, out);
+  return rc ? rc : status();
+}
+
+int direct_init_launch(const int *var, const int *var_ptr, const float *c, float *lam, long long Od, cudaStream_t stream) {
+  if (Od == 0) return 0;
+  direct_init_kernel<<<grid_for(Od), 256, 0, stream>>>(var, var_ptr, c, lam, Od);
+  return status();
+}
+
+int direct_pending_launch(const int *home, const int *ref, const int *var_ptr, const float *d, long long ext0, float *P, int n,
+                          cudaStream_t stream) {
+  if (n == 0) return 0;
+  direct_pending_kernel<<<grid_for(n), 256, 0, stream>>>(home, ref, var_ptr, d, ext0, P, n);
+  return status();
+}
+
+int direct_set_pending_launch(const int *home, const int *var_ptr, const float *P, long long ext0, float *d, int n,
+                              cudaStream_t stream) {
+  if (n == 0) return 0;
+  direct_set_pending_kernel<<<grid_for(n), 256, 0, stream>>>(home, var_ptr, P, ext0, d, n);
+  return status();
+}
+
+int direct_scatter_launch(const DirectParams &p, long long Od, float *out, bool fold, cudaStream_t stream) {
+  if (Od == 0) return 0;
+  direct_scatter_kernel<<<grid_for(Od), 256, 0, stream>>>(p, Od, out, fold);
+  return status();
+}
+
+int direct_gather_launch(const float *in, const long long *csr, float *lam, long long Od, cudaStream_t stream) {
+  if (Od == 0) return 0;
+  direct_gather_kernel<<<grid_for(Od), 256, 0, stream>>>(in, csr, lam, Od);
+  return status();
+}
+
+}  // namespace bdd

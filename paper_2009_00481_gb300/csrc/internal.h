@@ -239,6 +239,135 @@ inline int layout_key(int width, int depth) { return natural_class(width) * kDep
 int build_layout(const HostBDDs &H, Layout *L, bool lanes2 = false, const int *class_of_key = nullptr,
                  const int *var_deg = nullptr);
 
+// ---------------------------------------------------------------------------------------
+// Direct plan (plain solvers with the default options): no pending passes between the sweeps.
+// A sweep records its differences where the next sweep finds them and forms the pending share of
+// every occurrence itself, from the differences of the variable's other occurrences:
+//   - a variable in one or two rows: the difference is stored at the occurrence, and the share is
+//     its own difference, or half the sum of its own and its mate's;
+//   - a variable in more rows: its differences lie next to each other in a group of 4, 8, 16 or
+//     32 values behind the occurrences (unused ones 0), read with 16-byte loads and added in
+//     ascending row order -- the additions of the pending pass, so the same bits;
+//   - a variable in more than kGatherMax rows: a small kernel, one warp per such variable, sums
+//     its values after each sweep.
+// A forward sweep reads the differences of the backward sweep before it and the other way
+// round, so the two kinds are kept in two arrays.  The bound of an iteration is summed by the
+// forward sweep of the next one (or by a pass of its own after the last).
+//
+// Occurrences lie in rectangles: a tile of G BDDs and depth D holds D x G of them, layer-major, the
+// BDDs that end earlier padded (no arcs, cost 0, csr -1), so a lane finds its occurrences without
+// node offsets or depths.
+//
+// ref of an occurrence: >= 0: the occurrence itself (one row) or the variable's other one (two
+// rows).  Negative: bits 28-30 hold k, bits 0-27 the occurrence's place among the grouped values;
+// k = 0..5 a variable in 3 + k rows, kRefMid one in 9..16, kRefLong one in 17..32, or a heavy one
+// (ext_deg tells; 0 is heavy).
+// ---------------------------------------------------------------------------------------
+constexpr int kGatherMax = 32;
+constexpr int kRefMid = 6, kRefLong = 7;
+constexpr int kRefShift = 28;
+constexpr unsigned kRefPlace = (1u << kRefShift) - 1u;
+__host__ __device__ inline int ref_capacity(int k) { return k < 2 ? 4 : k < kRefMid ? 8 : k == kRefMid ? 16 : 32; }
+constexpr int kLaneRegDepth = 10;   // lane tiles up to this depth run in registers ...
+constexpr int kLaneDeepDepth = 32;  // ... up to this one (and those with a variable in more than 8
+                                    // rows, whose longer sums would cost every tile registers) from
+                                    // shared memory: kTileDeep is set in the tile's BDD count
+constexpr int kTileDeep = 64;
+constexpr int kCoopDepth = 6;
+constexpr int kTileChain = 256;   // in a tile's last word beside its depth: all of its BDDs have that
+constexpr int kTileDepth = 255;   // depth, and chain layers (kDirectChain) between first and last
+constexpr int kTileMaskShift = 9;  // above: a bit for each of the first layers with grouped values
+// lane codes of the direct plan: an arc (2 bits, as in lane_code) is 0 or 1 (that node of the next
+// layer; 0 also for top, which only a last layer's arcs reach) or kDirectBot
+constexpr unsigned kDirectBot = 2;
+constexpr unsigned kDirectNoNode1 = 0xA0u;  // both arcs of node 1 to bot: a one-node layer
+constexpr unsigned char kDirectPad = 0xA8;  // padding: node 0's 0-arc to node 0, the others to bot
+// node 0's arcs to nodes 0 and 1, node 1's to node 1 and bot
+constexpr unsigned kDirectChain = 0u | 1u << 2 | 1u << 4 | kDirectBot << 6;
+// shared memory per layer of a deep lane tile: two messages, multiplier, share, ref, code per lane
+constexpr int kLaneLayerBytes = 32 * (8 + 4 + 4 + 4 + 1);
+
+struct DirectLayout {
+  hvec<int> bdd_perm, bdd_depth;  // as in Layout
+  hvec<int> tile;                 // [4 tiles] first occurrence, first BDD, BDDs (| kTileDeep), depth (| kTileChain, ...)
+  int class_tile_off[kWarpClasses + 2] = {0};
+  int n_tiles = 0;
+  long long Od = 0;   // occurrences with padding
+  long long ext = 0;  // grouped values
+  int deep_depth = 0;  // deepest tile with kTileDeep
+  bool chains = false;  // every tile has kTileChain and not kTileDeep
+  hvec<unsigned char> code;  // [Od] lane codes (padding: no arcs)
+  hvec<int> ref;             // [Od]
+  hvec<long long> csr;       // [Od], -1: padding
+  hvec<int> var;             // [Od], -1: padding
+  hvec<int> occ_of_canon;    // canonical occurrence -> occurrence
+  hvec<int> var_ptr;         // [n + 1] occurrences of each variable (degrees)
+  hvec<int> home;            // [n] ref-style place of the variable's first difference (0: none)
+  hvec<unsigned char> ext_deg;  // [ext / 4] degree of the group each 4 values belong to (0: heavy)
+  hvec<int> heavy;           // [4 heavy] variable, first grouped value, rows, 0
+  hvec<int> heavy_of;        // [ext - heavy0] index of the heavy variable at a grouped value
+  long long heavy0 = 0;
+};
+
+// BDD_OK, BDD_ETOOBIG when the plan does not fit this instance (the caller then takes the general
+// layout), or BDD_EINVAL
+int build_direct_layout(const HostBDDs &H, DirectLayout *L, const int *var_deg);
+
+struct DirectParams {
+  const int4 *tile;
+  int n_tiles;
+  const unsigned char *code;
+  const int *ref;
+  const long long *csr;
+  float *lam;
+  const float *din;   // differences of the sweep before (occurrences, then grouped values)
+  float *dout;        // differences of this sweep
+  const float *ein;   // grouped values of din (din + n_occ)
+  const unsigned char *ext_deg;
+  const int *heavy_of;
+  const float2 *heavy;  // pending sum and share of every heavy variable
+  int heavy0;
+  int deep_depth;     // deepest tile with kTileDeep, 0: none
+  int chains;         // every tile is a chain tile that runs in registers
+  int n_coop;         // the first n_coop tiles take a block each (all of them kTileDeep)
+  int warp_depth;     // layers of shared memory per warp of the other blocks
+  float omega;
+  float *bdd_E;
+  float *out_m0, *out_m1;  // folded pass
+  double *partial;    // [blocks] bound partials
+  int sum_bound;      // forward update: add up the bound of the iteration before
+  int *error;
+  long long n_diff, n_csr, n_bdd, n_occ;  // extents (checked build)
+  // bound partials of the forward sweep before, finished by a block of this backward sweep
+  const double *fin_partial;
+  int fin_nblocks;
+  int *iter_ctr;
+  double *trace;
+  int trace_cap;
+  const double *empty_const;
+  unsigned *ticket;   // bound pass: the last block to arrive finishes the sum
+  int pdl_early;
+};
+enum DirectMode : int {
+  kDirectUpdate = 0,  // one sweep
+  kDirectEnergy = 1,  // E^j and, with sum_bound, the bound
+  kDirectFolded = 2,  // min-marginals at multipliers plus shares
+};
+// grid: blocks of kBlockThreads that take the tiles in turn (a backward update adds one block)
+int direct_launch(bool forward, int mode, const DirectParams &p, int grid, size_t smem, cudaStream_t stream);
+int direct_resident_blocks(bool chains, size_t smem, int *blocks);
+int direct_set_smem(size_t smem);
+int heavy_launch(const int4 *heavy, int n_heavy, const float *ein, float2 *out, cudaStream_t stream);
+int direct_init_launch(const int *var, const int *var_ptr, const float *c, float *lam, long long Od, cudaStream_t stream);
+// P[i] from the differences of the last backward sweep / those differences from P (the rest 0)
+int direct_pending_launch(const int *home, const int *ref, const int *var_ptr, const float *d, long long ext0, float *P, int n,
+                          cudaStream_t stream);
+int direct_set_pending_launch(const int *home, const int *var_ptr, const float *P, long long ext0, float *d, int n,
+                              cudaStream_t stream);
+// out[csr] = lam (+ share when fold)
+int direct_scatter_launch(const DirectParams &p, long long Od, float *out, bool fold, cudaStream_t stream);
+int direct_gather_launch(const float *in, const long long *csr, float *lam, long long Od, cudaStream_t stream);
+
 // Fused pending pass of an update sweep (the per-phase plan without separate pending kernels).
 // At the end of its tile every occurrence counts its variable down; the visit that brings the
 // count to zero is the variable's last in this sweep, so all of its slots are final: it forms

@@ -83,11 +83,18 @@ def dist_env():
 # algorithmic bytes per kernel launch (minimum traffic of the slab layout: every array a kernel
 # needs, touched once)
 # ------------------------------------------------------------------------------------------
-def graph_launches(iters: int) -> int:
+def direct_plan(s) -> bool:
+    """Whether a solver built with the default options runs the direct plan: every BDD in lane tiles
+    whose sweeps form their own shares (no pending passes)."""
+    return bool(getattr(s, "lanes", 0)) and s.lane_O == s.O and s.schedule == 1 and s.staging == 0
+
+
+def graph_launches(iters: int, s=None) -> int:
     """Kernels the per-phase schedule launches for `iters` iterations: four per iteration (two
-    sweeps, two pending passes), plus the one-warp kernel that finishes the last bound of each
-    captured chain (chains of 8 iterations, then single iterations)."""
-    return 4 * iters + iters // 8 + iters % 8
+    sweeps, two pending passes), two with the direct plan (the workloads have no variable in more
+    than 32 rows there), plus the kernel that finishes the last bound of each captured chain
+    (chains of 8 iterations, then single iterations)."""
+    return (2 if s is not None and direct_plan(s) else 4) * iters + iters // 8 + iters % 8
 
 
 def algorithmic_bytes(kind: str, N: int, O: int, n: int, nb: int, lane_N: int = 0, lane_O: int = 0) -> int:
@@ -112,8 +119,21 @@ def algorithmic_bytes(kind: str, N: int, O: int, n: int, nb: int, lane_N: int = 
     raise ValueError(kind)
 
 
+def direct_bytes(kind: str, s) -> int:
+    """Bytes a sweep of the direct plan must move: per occurrence ref 4, multiplier read and write 8,
+    difference read and write 8 (a mate's difference is another occurrence's own); per BDD the
+    codes of its first and last layer 2 (chain layers need none) and, on the backward sweep, the
+    root value 4.  The bound pass after a chain reads the same without writing."""
+    per = {"fwd": 20 * s.O + 2 * s.nb, "pending": 0, "bwd": 20 * s.O + 6 * s.nb, "pending_bound": 12 * s.O + 6 * s.nb}
+    if kind == "iteration":
+        return per["fwd"] + per["bwd"] + per["pending_bound"] // 8
+    return per[kind]
+
+
 def solver_bytes(kind: str, s) -> int:
     """algorithmic_bytes of a solver's layout."""
+    if direct_plan(s):
+        return direct_bytes(kind, s)
     return algorithmic_bytes(kind, s.N, s.O, s.n, s.nb, getattr(s, "lane_N", 0), getattr(s, "lane_O", 0))
 
 
@@ -129,7 +149,10 @@ def staging_of(s) -> dict:
 
 def sweep_kernel_name(kind: str, s) -> str:
     """The sweep kernel as the solver runs it: lane tiles (if its layout has them) and the
-    staging of its other warp tiles."""
+    staging of its other warp tiles; the direct plan's sweeps."""
+    if direct_plan(s):
+        return {"fwd": "direct_kernel<forward, update>", "bwd": "direct_kernel<backward, update>",
+                "pending": "none (shares formed by the sweeps)", "pending_bound": "direct_kernel<energy> (bound)"}[kind]
     st = staging_of(s)
     lanes = "lane tiles + " if getattr(s, "lanes", 0) else ""
     return {"fwd": f"sweep_kernel<forward, update> ({lanes}{st['forward']})",
@@ -381,12 +404,13 @@ def timed_steps(torch, s, inst, iters, steps, warmup, stream, trace):
 
 def roofline_of(s, iters, kms, peak, peak_kind, workload, label=None):
     """Roofline of the dominant per-phase kernel from the kernel-by-kernel event timings."""
-    dom = int(np.argmax(kms))
+    dom = int(np.argmax(kms[:3] if direct_plan(s) else kms))
     abytes = solver_bytes(KINDS[dom], s)
     per_launch_ms = float(kms[dom] / iters)
     achieved = abytes / (per_launch_ms / 1e3) / 1e9
     iter_bytes = solver_bytes("iteration", s)
-    iter_ms = float(kms.sum() / iters)
+    # direct plan: the bound pass, timed after every iteration here, runs once per chain of 8
+    iter_ms = float(kms[0] + kms[2] + kms[3] / 8) / iters if direct_plan(s) else float(kms.sum() / iters)
     name = sweep_kernel_name(KINDS[dom], s)
     out = {"bound": "hbm", "kernel": name, "achieved": achieved, "peak": peak, "peak_kind": peak_kind,
            "unit": "GB/s", "frac": achieved / peak, "traffic": dram_traffic(workload, name, s.N),
@@ -539,7 +563,7 @@ def run_batch(args):
         "plain_loop": None if plain is None else {k: v for k, v in plain.items()
                                                   if k not in ("traces", "ms_per_solver")},
         "forms": forms,
-        "gpu_launches": args.steps * graph_launches(iters),
+        "gpu_launches": args.steps * graph_launches(iters, s),
         "schedule": "persistent" if s.schedule == 0 else "per-phase graphs",
         "staging": staging_of(s),
         "clocks": clocks,
@@ -806,7 +830,7 @@ def run_single(args):
                              "ms": ms * kk / iters if kk else None},
            "cpu_baseline": {"value": 2 * s.N * iters / osec, "unit": UNIT, "cores": 1, "kind": "oracle",
                             "sample": f"full {CONFIG_NAMES[k]} instance, {iters} iterations, FP64 single thread"},
-           "gpu_launches": args.steps * graph_launches(iters), "staging": staging_of(s), "clocks": clocks}
+           "gpu_launches": args.steps * graph_launches(iters, s), "staging": staging_of(s), "clocks": clocks}
     print(json.dumps(out), flush=True)
 
 

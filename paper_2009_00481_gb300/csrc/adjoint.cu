@@ -370,221 +370,274 @@ __device__ void bwd_adjoint_tile(const AdjParams &a, int tile) {
 // before 1-arc), so the sums do not depend on timing.  Reductions over a layer go warp by warp
 // and then over the warps in order; the soft minima of a layer are the forward sweep's
 // group_agg2 reduction (the same order, so the same values).
+//
+// The layers are one dependent chain, so what a layer waits for decides: the per-layer values are
+// staged in shared memory once and the results written back after the last layer, a node's arcs and
+// messages are loaded two layers ahead and its targets' messages one, the exchanges alternate
+// between two buffers (one barrier each), and a pull visits a node's predecessors (their places
+// come with its record, SweepParams::node_rec) instead of scanning the layer.
 // ---------------------------------------------------------------------------------------
 struct BlockAdjSmem {
-  float G[kBlockThreads];   // adjoints of layer l + 1's nodes (pull from children)
-  float F[kBlockThreads];   // their messages
-  int2 arcs[kBlockThreads]; // arcs of layer l
-  float c0[kBlockThreads], c1[kBlockThreads];  // contributions along the 0- and 1-arcs
-  float red[kWarpsPerBlock];
-  float2 red2[kWarpsPerBlock];
+  float G[2][kBlockThreads];   // adjoints of a layer's nodes (pull from children)
+  float F[2][kBlockThreads];   // their messages
+  int2 arcs[2][kBlockThreads]; // arcs of a layer (layouts without records)
+  float c0[2][kBlockThreads], c1[2][kBlockThreads];  // contributions along the 0- and 1-arcs
+  float4 red[2][kWarpsPerBlock];  // the warps' sums and soft minima
 };
+// per-layer values of a block tile in dynamic shared memory
+struct BlockLayers {
+  int *off;                            // [depth + 1] node offsets
+  float *lam_s, *shr_s, *lam2;         // multipliers, shares, updated multipliers
+  float *g_lam, *g_diff;               // adjoints of the layer's outputs; g_lam becomes the input's
+  float4 *part;                        // the warps' sums of the second walk
+};
+__host__ __device__ inline size_t block_layers_bytes(int depth_buf) { return 40 * (size_t)depth_buf + 32; }
 
-// sum over the block, the same value on every thread (warp sums, then the warps in order)
-__device__ __forceinline__ float block_sum_f(float v, float *red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  v = team_sum<32>(v);
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  float r = red[0];
-#pragma unroll
-  for (int t = 1; t < kWarpsPerBlock; ++t) r += red[t];
-  __syncthreads();
-  return r;
-}
-
-// soft minima of a and b over the block (group_agg2 of the sweeps, the same order)
-__device__ __forceinline__ float2 block_softmin2(float a, float b, const SweepParams &p, float2 *red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  a = team_agg<32, true>(a, p);
-  b = team_agg<32, true>(b, p);
-  if (lane == 0) red[warp] = make_float2(a, b);
-  __syncthreads();
-  float2 r = red[0];
-#pragma unroll
-  for (int t = 1; t < kWarpsPerBlock; ++t) {
-    r.x = soft_min(r.x, red[t].x, p.alpha, p.inv_alpha);
-    r.y = soft_min(r.y, red[t].y, p.alpha, p.inv_alpha);
+__device__ __forceinline__ BlockLayers block_layers(char *smem, const AdjParams &a, int occ0, int depth) {
+  const SweepParams &p = a.sp;
+  const int n = p.block_depth_buf;
+  BlockLayers L;
+  L.part = reinterpret_cast<float4 *>(smem);
+  L.lam_s = reinterpret_cast<float *>(L.part + n);
+  L.shr_s = L.lam_s + n;
+  L.lam2 = L.shr_s + n;
+  L.g_lam = L.lam2 + n;
+  L.g_diff = L.g_lam + n;
+  L.off = reinterpret_cast<int *>(L.g_diff + n);
+  for (int l = threadIdx.x; l <= depth; l += kBlockThreads) L.off[l] = p.occ_node_off[occ0 + l];
+  for (int l = threadIdx.x; l < depth; l += kBlockThreads) {
+    const int o = occ0 + l;
+    L.lam_s[l] = a.lam_s[o];
+    L.shr_s[l] = a.shr_s[o];
+    L.lam2[l] = a.lam2[o];
+    L.g_lam[l] = a.g_out_lam[o];
+    L.g_diff[l] = a.g_out_delta[p.occ_slot[o]];
   }
   __syncthreads();
-  return r;
+  return L;
+}
+// g_in_lam and g_shr of the tile: the first walk's value, and with the second walk's sums added
+__device__ __forceinline__ void block_write(const AdjParams &a, const BlockLayers &L, int occ0, int depth) {
+  __syncthreads();
+  for (int l = threadIdx.x; l < depth; l += kBlockThreads) {
+    const float4 q = L.part[l];
+    a.g_shr[occ0 + l] = L.g_lam[l];
+    a.g_in_lam[occ0 + l] = L.g_lam[l] + (q.x + q.y + q.z + q.w);  // the warps in order
+  }
 }
 
-// node c (< w_next) of layer l + 1, starting at node0n: the sum of the contributions along the
-// arcs of layer l's w nodes that enter it (S.arcs, S.c0, S.c1 filled before a barrier)
-__device__ __forceinline__ float pull_sum(const BlockAdjSmem &S, int w, int node0n, int c) {
-  const int v = node0n + c;
+// a node of a layer: its arcs, two per-node values, its predecessors (node_rec); none past the layer
+struct BlockNode {
+  int2 lh;
+  float x, y;
+  unsigned pred;
+  bool has;
+};
+__device__ __forceinline__ BlockNode block_node(const AdjParams &a, const BlockLayers &L, int l, int depth, const float *X,
+                                                const float *Y) {
+  BlockNode q{make_int2(kNone, kNone), 0.f, 0.f, 0u, false};
+  if (l < 0 || l >= depth) return q;
+  const int n = L.off[l] + threadIdx.x;
+  q.has = n < L.off[l + 1];
+  if (q.has) {
+    q.lh = a.sp.lohi[n];
+    q.x = X[n];
+    if (Y) q.y = Y[n];
+    if (a.sp.node_rec) q.pred = a.sp.node_rec[n - a.sp.rec0].y;
+  }
+  return q;
+}
+
+// the sum of the contributions along the arcs of layer l's w nodes that enter node v of the next one
+__device__ __forceinline__ float pull_sum(const AdjParams &a, const BlockAdjSmem &S, int b, int w, int v, unsigned pred) {
   float acc = 0.f;
-  for (int u = 0; u < w; ++u) {
-    const int2 q = S.arcs[u];
-    if (q.x == v) acc += S.c0[u];
-    if (q.y == v) acc += S.c1[u];
+  if (!a.sp.node_rec) {
+    for (int u = 0; u < w; ++u) {
+      const int2 q = S.arcs[b][u];
+      if (q.x == v) acc += S.c0[b][u];
+      if (q.y == v) acc += S.c1[b][u];
+    }
+    return acc;
+  }
+  PredRuns r(pred, a.sp.block_buf);
+  while (r.more()) {
+    const int u = r.node();
+    acc += r.take() ? S.c1[b][u] : S.c0[b][u];
   }
   return acc;
 }
 
-__device__ void fwd_adjoint_block(const AdjParams &a, int tile, BlockAdjSmem &S) {
+// sum of v, soft minima of x and y over the block: one barrier (two buffers)
+__device__ __forceinline__ float3 block_sum_softmin2(float v, float x, float y, const SweepParams &p, float4 *red) {
+  v = team_sum<32>(v);
+  x = team_agg<32, true>(x, p);
+  y = team_agg<32, true>(y, p);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float4(v, x, y, 0.f);
+  __syncthreads();
+  float4 r = red[0];
+#pragma unroll
+  for (int t = 1; t < kWarpsPerBlock; ++t) {
+    const float4 q = red[t];
+    r.x += q.x;
+    r.y = soft_min(r.y, q.y, p.alpha, p.inv_alpha);
+    r.z = soft_min(r.z, q.z, p.alpha, p.inv_alpha);
+  }
+  return make_float3(r.x, r.y, r.z);
+}
+__device__ __forceinline__ void warp_part(float4 *part, float v) {
+  v = team_sum<32>(v);
+  if ((threadIdx.x & 31) == 0) reinterpret_cast<float *>(part)[threadIdx.x >> 5] = v;
+}
+
+__device__ void fwd_adjoint_block(const AdjParams &a, int tile, BlockAdjSmem &S, char *smem) {
   const SweepParams &p = a.sp;
   const float ia = p.inv_alpha;
   const int gt = threadIdx.x;
   const int bdd = p.tile_bdd0[tile], occ0 = p.tile_occ0[tile], depth = p.bdd_depth[bdd];
+  const BlockLayers L = block_layers(smem, a, occ0, depth);
+  const int *off = L.off;
   // descending layers: adjoint of fm_l pulled from the children, the marginal terms, their
   // contributions to the starting backward messages of layer l + 1 (g_node)
+  BlockNode c = block_node(a, L, depth - 1, depth, a.msg_new, nullptr), n1 = block_node(a, L, depth - 2, depth, a.msg_new, nullptr);
+  float cb0 = target_msg(a.msg_pre, c.lh.x), cb1 = target_msg(a.msg_pre, c.lh.y);
+  unsigned pred_next = 0u;  // of this thread's node in layer l + 1
   for (int l = depth - 1; l >= 0; --l) {
-    const int o = occ0 + l;
-    const int node0 = p.occ_node_off[o], w = p.occ_node_off[o + 1] - node0;
+    const BlockNode q = c;
+    const float b0 = q.has ? cb0 : inf(), b1 = q.has ? cb1 : inf();
+    c = n1;
+    cb0 = target_msg(a.msg_pre, c.lh.x);
+    cb1 = target_msg(a.msg_pre, c.lh.y);
+    n1 = block_node(a, L, l - 2, depth, a.msg_new, nullptr);
+    const int buf = l & 1, w = off[l + 1] - off[l];
     const bool nxt = l + 1 < depth;
-    const int node0n = node0 + w, wn = nxt ? p.occ_node_off[o + 2] - node0n : 0;
-    const bool has = gt < w;
-    int2 lh = make_int2(kNone, kNone);
-    float f = inf();
-    if (has) {
-      lh = p.lohi[node0 + gt];
-      f = a.msg_new[node0 + gt];
-    }
-    const float lam1 = a.lam_s[o] + a.shr_s[o], lam2 = a.lam2[o];
+    const int node0n = off[l + 1], wn = nxt ? off[l + 2] - node0n : 0;
+    const float f = q.has ? q.x : inf();
+    const float lam1 = L.lam_s[l] + L.shr_s[l], lam2 = L.lam2[l];
     float G = 0.f, g_theta = 0.f;
-    if (has && nxt) {  // S.G, S.F: layer l + 1 (written at the end of the previous step)
-      if (lh.x >= 0) G += S.G[lh.x - node0n] * weight(f, S.F[lh.x - node0n], ia);
-      if (lh.y >= 0) {
-        g_theta = S.G[lh.y - node0n] * weight(f + lam2, S.F[lh.y - node0n], ia);
+    if (q.has && nxt) {  // layer l + 1 (written by the previous step, before its last barrier)
+      const float *Gn = S.G[buf ^ 1], *Fn = S.F[buf ^ 1];
+      if (q.lh.x >= 0) G += Gn[q.lh.x - node0n] * weight(f, Fn[q.lh.x - node0n], ia);
+      if (q.lh.y >= 0) {
+        g_theta = Gn[q.lh.y - node0n] * weight(f + lam2, Fn[q.lh.y - node0n], ia);
         G += g_theta;
       }
     }
-    const float G_lam2 = a.g_out_lam[o] + block_sum_f(g_theta, S.red);
-    const float b0 = has ? target_msg(a.msg_pre, lh.x) : inf();
-    const float b1 = has ? target_msg(a.msg_pre, lh.y) : inf();
-    const float a0 = has ? f + b0 : inf(), a1 = has ? f + lam1 + b1 : inf();
-    const float2 mm = block_softmin2(a0, a1, p, S.red2);
-    const bool finite = mm.x < inf() && mm.y < inf();
-    const float gd = finite ? p.omega * (a.g_out_delta[p.occ_slot[o]] - G_lam2) : 0.f;
-    const float p0 = weight(a0, mm.x, ia), p1 = weight(a1, mm.y, ia);
+    const float a0 = q.has ? f + b0 : inf(), a1 = q.has ? f + lam1 + b1 : inf();
+    const float3 r = block_sum_softmin2(g_theta, a0, a1, p, S.red[buf]);
+    const float G_lam2 = L.g_lam[l] + r.x;
+    const bool finite = r.y < inf() && r.z < inf();
+    const float gd = finite ? p.omega * (L.g_diff[l] - G_lam2) : 0.f;
+    const float p0 = weight(a0, r.y, ia), p1 = weight(a1, r.z, ia);
     G += -gd * p0 + gd * p1;
-    if (gt == 0) {
-      a.g_in_lam[o] = G_lam2 + gd;
-      a.g_shr[o] = G_lam2 + gd;
-    }
-    if (gt < kBlockThreads) {
-      S.arcs[gt] = nxt ? lh : make_int2(kNone, kNone);
-      S.c0[gt] = -gd * p0;
-      S.c1[gt] = gd * p1;
-    }
+    S.arcs[buf][gt] = nxt ? q.lh : make_int2(kNone, kNone);
+    S.c0[buf][gt] = -gd * p0;
+    S.c1[buf][gt] = gd * p1;
+    S.G[buf][gt] = q.has ? G : 0.f;
+    S.F[buf][gt] = f;
     __syncthreads();
-    if (gt < wn) a.g_node[node0n + gt] = pull_sum(S, w, node0n, gt);
-    __syncthreads();  // S.G / S.F of layer l + 1 no longer read
-    S.G[gt] = has ? G : 0.f;
-    S.F[gt] = f;
-    __syncthreads();
+    if (gt == 0) L.g_lam[l] = G_lam2 + gd;  // (everyone has read the layer's entry)
+    if (gt < wn) a.g_node[node0n + gt] = pull_sum(a, S, buf, w, node0n + gt, pred_next);
+    pred_next = q.pred;
   }
+  __syncthreads();
   // ascending layers: the starting backward messages bmp_l(v) = softmin(bmp_{l+1}(lo),
   // lam_l + bmp_{l+1}(hi)), adjoints flowing from layer l to layer l + 1
   float carry = 0.f;
+  c = block_node(a, L, 0, depth, a.msg_pre, nullptr);
+  n1 = block_node(a, L, 1, depth, a.msg_pre, a.g_node);
+  cb0 = target_msg(a.msg_pre, c.lh.x);
+  cb1 = target_msg(a.msg_pre, c.lh.y);
   for (int l = 0; l < depth; ++l) {
-    const int o = occ0 + l;
-    const int node0 = p.occ_node_off[o], w = p.occ_node_off[o + 1] - node0;
+    const BlockNode q = c;
+    const float b0 = q.has ? cb0 : inf(), b1 = q.has ? cb1 : inf();
+    c = n1;
+    cb0 = target_msg(a.msg_pre, c.lh.x);
+    cb1 = target_msg(a.msg_pre, c.lh.y);
+    n1 = block_node(a, L, l + 2, depth, a.msg_pre, a.g_node);
+    const int buf = l & 1, w = off[l + 1] - off[l];
     const bool nxt = l + 1 < depth;
-    const int node0n = node0 + w, wn = nxt ? p.occ_node_off[o + 2] - node0n : 0;
-    const bool has = gt < w;
-    int2 lh = make_int2(kNone, kNone);
-    float bn = inf(), Gb = 0.f;
-    if (has) {
-      lh = p.lohi[node0 + gt];
-      bn = a.msg_pre[node0 + gt];
-      if (l >= 1) Gb = a.g_node[node0 + gt] + carry;
-    }
-    const float lam = a.lam_s[o];
-    const float b0 = has ? target_msg(a.msg_pre, lh.x) : inf();
-    const float b1 = has ? target_msg(a.msg_pre, lh.y) : inf();
-    const float q0 = has ? weight(b0, bn, ia) : 0.f;
-    const float q1 = has ? weight(lam + b1, bn, ia) : 0.f;
-    const float gl = block_sum_f(Gb * q1, S.red);
-    if (gt == 0) a.g_in_lam[o] += gl;
-    S.arcs[gt] = nxt ? lh : make_int2(kNone, kNone);
-    S.c0[gt] = Gb * q0;
-    S.c1[gt] = Gb * q1;
+    const int node0n = off[l + 1], wn = nxt ? off[l + 2] - node0n : 0;
+    const float bn = q.has ? q.x : inf(), Gb = q.has && l >= 1 ? q.y + carry : 0.f;
+    const float q0 = q.has ? weight(b0, bn, ia) : 0.f;
+    const float q1 = q.has ? weight(L.lam_s[l] + b1, bn, ia) : 0.f;
+    warp_part(&L.part[l], Gb * q1);
+    S.arcs[buf][gt] = nxt ? q.lh : make_int2(kNone, kNone);
+    S.c0[buf][gt] = Gb * q0;
+    S.c1[buf][gt] = Gb * q1;
     __syncthreads();
-    carry = gt < wn ? pull_sum(S, w, node0n, gt) : 0.f;
-    __syncthreads();
+    carry = gt < wn ? pull_sum(a, S, buf, w, node0n + gt, c.pred) : 0.f;
   }
+  block_write(a, L, occ0, depth);
 }
 
-__device__ void bwd_adjoint_block(const AdjParams &a, int tile, BlockAdjSmem &S) {
+__device__ void bwd_adjoint_block(const AdjParams &a, int tile, BlockAdjSmem &S, char *smem) {
   const SweepParams &p = a.sp;
   const float ia = p.inv_alpha;
   const int gt = threadIdx.x;
   const int bdd = p.tile_bdd0[tile], occ0 = p.tile_occ0[tile], depth = p.bdd_depth[bdd];
+  const BlockLayers L = block_layers(smem, a, occ0, depth);
+  const int *off = L.off;
   // ascending layers (the reverse of the sweep): the adjoint of bmn_l (seeded at the root with
   // gE) through the backward step and, with the marginal terms, on to layer l + 1; the marginal
   // terms' adjoints of the starting forward messages go to g_node
-  float carry = 0.f;
+  float carry = gt == 0 && a.gE ? (float)*a.gE : 0.f;
+  BlockNode c = block_node(a, L, 0, depth, a.msg_pre, a.msg_new), n1 = block_node(a, L, 1, depth, a.msg_pre, a.msg_new);
+  float cb0 = target_msg(a.msg_new, c.lh.x), cb1 = target_msg(a.msg_new, c.lh.y);
   for (int l = 0; l < depth; ++l) {
-    const int o = occ0 + l;
-    const int node0 = p.occ_node_off[o], w = p.occ_node_off[o + 1] - node0;
+    const BlockNode q = c;
+    const float b0 = q.has ? cb0 : inf(), b1 = q.has ? cb1 : inf();
+    c = n1;
+    cb0 = target_msg(a.msg_new, c.lh.x);
+    cb1 = target_msg(a.msg_new, c.lh.y);
+    n1 = block_node(a, L, l + 2, depth, a.msg_pre, a.msg_new);
+    const int buf = l & 1, w = off[l + 1] - off[l];
     const bool nxt = l + 1 < depth;
-    const int node0n = node0 + w, wn = nxt ? p.occ_node_off[o + 2] - node0n : 0;
-    const bool has = gt < w;
-    int2 lh = make_int2(kNone, kNone);
-    float fp = inf(), bn = inf(), Gbn = 0.f;
-    if (has) {
-      lh = p.lohi[node0 + gt];
-      fp = a.msg_pre[node0 + gt];
-      bn = a.msg_new[node0 + gt];
-      Gbn = l == 0 ? (gt == 0 && a.gE ? (float)*a.gE : 0.f) : carry;
-    }
-    const float lam1 = a.lam_s[o] + a.shr_s[o], lam2 = a.lam2[o];
-    const float b0 = has ? target_msg(a.msg_new, lh.x) : inf();
-    const float b1 = has ? target_msg(a.msg_new, lh.y) : inf();
-    const float q0 = has ? weight(b0, bn, ia) : 0.f;
-    const float q1 = has ? weight(lam2 + b1, bn, ia) : 0.f;
-    const float G_lam2 = a.g_out_lam[o] + block_sum_f(Gbn * q1, S.red);
-    const float a0 = has ? fp + b0 : inf(), a1 = has ? fp + lam1 + b1 : inf();
-    const float2 mm = block_softmin2(a0, a1, p, S.red2);
-    const bool finite = mm.x < inf() && mm.y < inf();
-    const float gd = finite ? p.omega * (a.g_out_delta[p.occ_slot[o]] - G_lam2) : 0.f;
-    const float p0 = weight(a0, mm.x, ia), p1 = weight(a1, mm.y, ia);
-    if (has) a.g_node[node0 + gt] = -gd * p0 + gd * p1;
-    if (gt == 0) {
-      a.g_in_lam[o] = G_lam2 + gd;
-      a.g_shr[o] = G_lam2 + gd;
-    }
-    S.arcs[gt] = nxt ? lh : make_int2(kNone, kNone);
-    S.c0[gt] = Gbn * q0 - gd * p0;
-    S.c1[gt] = Gbn * q1 + gd * p1;
+    const int node0n = off[l + 1], wn = nxt ? off[l + 2] - node0n : 0;
+    const float fp = q.has ? q.x : inf(), bn = q.has ? q.y : inf(), Gbn = q.has ? carry : 0.f;
+    const float lam1 = L.lam_s[l] + L.shr_s[l], lam2 = L.lam2[l];
+    const float q0 = q.has ? weight(b0, bn, ia) : 0.f;
+    const float q1 = q.has ? weight(lam2 + b1, bn, ia) : 0.f;
+    const float a0 = q.has ? fp + b0 : inf(), a1 = q.has ? fp + lam1 + b1 : inf();
+    const float3 r = block_sum_softmin2(Gbn * q1, a0, a1, p, S.red[buf]);
+    const float G_lam2 = L.g_lam[l] + r.x;
+    const bool finite = r.y < inf() && r.z < inf();
+    const float gd = finite ? p.omega * (L.g_diff[l] - G_lam2) : 0.f;
+    const float p0 = weight(a0, r.y, ia), p1 = weight(a1, r.z, ia);
+    if (q.has) a.g_node[off[l] + gt] = -gd * p0 + gd * p1;
+    S.arcs[buf][gt] = nxt ? q.lh : make_int2(kNone, kNone);
+    S.c0[buf][gt] = Gbn * q0 - gd * p0;
+    S.c1[buf][gt] = Gbn * q1 + gd * p1;
     __syncthreads();
-    carry = gt < wn ? pull_sum(S, w, node0n, gt) : 0.f;
-    __syncthreads();
+    if (gt == 0) L.g_lam[l] = G_lam2 + gd;
+    carry = gt < wn ? pull_sum(a, S, buf, w, node0n + gt, c.pred) : 0.f;
   }
+  __syncthreads();
   // descending layers: the starting forward messages fmp_l(v) = softmin over in-arcs of
   // fmp_{l-1}(u) + theta, adjoints flowing from layer l + 1 back to layer l
+  c = block_node(a, L, depth - 1, depth, a.msg_pre, a.g_node);
+  n1 = block_node(a, L, depth - 2, depth, a.msg_pre, a.g_node);
   for (int l = depth - 1; l >= 0; --l) {
-    const int o = occ0 + l;
-    const int node0 = p.occ_node_off[o], w = p.occ_node_off[o + 1] - node0;
-    const bool nxt = l + 1 < depth;
-    const int node0n = node0 + w;
-    const bool has = gt < w;
-    int2 lh = make_int2(kNone, kNone);
-    float f = inf(), G = 0.f;
-    if (has) {
-      lh = p.lohi[node0 + gt];
-      f = a.msg_pre[node0 + gt];
-      G = a.g_node[node0 + gt];
-    }
-    const float lam = a.lam_s[o];
+    const BlockNode q = c;
+    c = n1;
+    n1 = block_node(a, L, l - 2, depth, a.msg_pre, a.g_node);
+    const int buf = l & 1, node0n = off[l + 1];
+    const float f = q.has ? q.x : inf();
+    float G = q.has ? q.y : 0.f;
     float g_theta = 0.f;
-    if (has && nxt) {
-      if (lh.x >= 0) G += S.G[lh.x - node0n] * weight(f, S.F[lh.x - node0n], ia);
-      if (lh.y >= 0) {
-        g_theta = S.G[lh.y - node0n] * weight(f + lam, S.F[lh.y - node0n], ia);
+    if (q.has && l + 1 < depth) {
+      const float *Gn = S.G[buf ^ 1], *Fn = S.F[buf ^ 1];
+      if (q.lh.x >= 0) G += Gn[q.lh.x - node0n] * weight(f, Fn[q.lh.x - node0n], ia);
+      if (q.lh.y >= 0) {
+        g_theta = Gn[q.lh.y - node0n] * weight(f + L.lam_s[l], Fn[q.lh.y - node0n], ia);
         G += g_theta;
       }
     }
-    const float gl = block_sum_f(g_theta, S.red);
-    if (gt == 0) a.g_in_lam[o] += gl;
-    __syncthreads();  // S.G / S.F of layer l + 1 no longer read
-    S.G[gt] = has ? G : 0.f;
-    S.F[gt] = f;
+    warp_part(&L.part[l], g_theta);
+    S.G[buf][gt] = q.has ? G : 0.f;
+    S.F[buf][gt] = f;
     __syncthreads();
   }
+  block_write(a, L, occ0, depth);
 }
 
 template <bool FWD>
@@ -623,10 +676,11 @@ __global__ void __launch_bounds__(kBlockThreads) sweep_adjoint_kernel(const AdjP
   const int tile = a.sp.class_tile_off[kWarpClasses] + ((int)blockIdx.x - a.sp.n_warp_blocks);
   if (tile >= a.sp.class_tile_off[kWarpClasses + 1]) return;  // uniform across the block
   __shared__ BlockAdjSmem S;
+  extern __shared__ __align__(16) char layers[];
   if (FWD)
-    fwd_adjoint_block(a, tile, S);
+    fwd_adjoint_block(a, tile, S, layers);
   else
-    bwd_adjoint_block(a, tile, S);
+    bwd_adjoint_block(a, tile, S, layers);
 }
 
 // Adjoint of the pending sums: share_o = P_i / |J_i| and P_i = sum of the previous sweep's
@@ -695,10 +749,16 @@ int launch_status() { return cudaGetLastError() == cudaSuccess ? 0 : -5; }
 
 int sweep_adjoint_launch(bool forward, const AdjParams &a, int grid, cudaStream_t stream) {
   if (grid <= 0) return 0;
+  const bool blocks = a.sp.class_tile_off[kWarpClasses + 1] > a.sp.class_tile_off[kWarpClasses];
+  const size_t smem = blocks ? block_layers_bytes(a.sp.block_depth_buf) : 0;
+  if (smem > 40 * 1024) {  // (the static buffers come on top)
+    const void *f = forward ? (const void *)sweep_adjoint_kernel<true> : (const void *)sweep_adjoint_kernel<false>;
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -5;
+  }
   if (forward)
-    sweep_adjoint_kernel<true><<<grid, kBlockThreads, 0, stream>>>(a);
+    sweep_adjoint_kernel<true><<<grid, kBlockThreads, smem, stream>>>(a);
   else
-    sweep_adjoint_kernel<false><<<grid, kBlockThreads, 0, stream>>>(a);
+    sweep_adjoint_kernel<false><<<grid, kBlockThreads, smem, stream>>>(a);
   return launch_status();
 }
 

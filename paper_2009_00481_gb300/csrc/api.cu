@@ -82,6 +82,8 @@ struct bdd_solver {
   int *d_occ_node_off = nullptr, *d_occ_var = nullptr;
   long long *d_occ_csr = nullptr;
   int2 *d_lohi = nullptr;
+  uint2 *d_node_rec = nullptr;           // one-barrier block tiles (SweepParams::node_rec)
+  int rec0 = 0;
   unsigned char *d_lane_code = nullptr;  // lane tiles: arcs of a layer in one byte per occurrence
   long long lane_O = 0, lane_N = 0;      // occurrences and nodes of the lane tiles
   float *d_fm = nullptr, *d_bm = nullptr, *d_lam = nullptr, *d_delta = nullptr;
@@ -242,6 +244,8 @@ struct bdd_solver {
     p.n_csr = nnz;
     p.n_bdd = nb;
     p.inv_alpha = alpha > 0.f ? 1.f / alpha : 0.f;
+    p.node_rec = d_node_rec;
+    p.rec0 = rec0;
     p.copy_val = d_mu_bar;
     p.split = npairs > 0 ? 1 : 0;
     return p;
@@ -771,8 +775,10 @@ int setup_device(bdd_solver *h, const Layout &L, const float *c, const CutTables
   const int heavy_blocks = (n_heavy + kReduceThreads / 32 - 1) / (kReduceThreads / 32);
   h->grid_reduce = std::max(1, std::min(std::max((range + kReduceThreads - 1) / kReduceThreads, heavy_blocks), 152 * 16));
   // the largest dynamic shared memory any staging variant's sweep launch asks for
-  h->smem = std::max(sweep_smem_bytes(h->block_buf, h->block_depth_buf, 0, h->lanes2, h->alpha > 0.f),
-                     sweep_smem_bytes(h->block_buf, h->block_depth_buf, 2, h->lanes2, h->alpha > 0.f));
+  // (smoothed solvers have a form of their own)
+  const bool fast = !L.node_rec.empty() && h->alpha == 0.f;
+  h->smem = std::max(sweep_smem_bytes(h->block_buf, h->block_depth_buf, 0, h->lanes2, h->alpha > 0.f, fast),
+                     sweep_smem_bytes(h->block_buf, h->block_depth_buf, 2, h->lanes2, h->alpha > 0.f, fast));
   h->smem_persist = persist_smem_bytes(h->block_buf, h->block_depth_buf);
   if (h->smem > 48 * 1024 && sweep_set_smem(h->smem)) return BDD_ECUDA;
   // programmatic dependent launch: each per-phase kernel lets its successor launch as soon as it
@@ -807,7 +813,7 @@ int setup_device(bdd_solver *h, const Layout &L, const float *c, const CutTables
   const long long ntiles = (long long)L.tile_bdd0.size();
   long long need = (O + 1) * 4 + O * 4 + O * 8 + N * 8 + 2 * N * 4 + 2 * O * 4 + 3 * (long long)n * 4 +
                    nb * 8 + 3 * ntiles * 4 + (n + 1) * 4 + O * 4 + h->grid_reduce * 8 + 1024 * 8 +
-                   (h->averaging == 1 ? O : 0) + (h->lanes2 ? O + kLaneCodePad : 0) + 4LL * (long long)(L.tile_win0.size() + L.win_node.size()) + (h->fused ? 12 * n + 8LL * (h->grid_sweep + h->grid_reduce) : 0) +
+                   (h->averaging == 1 ? O : 0) + 4LL * (long long)L.node_rec.size() + (h->lanes2 ? O + kLaneCodePad : 0) + 4LL * (long long)(L.tile_win0.size() + L.win_node.size()) + (h->fused ? 12 * n + 8LL * (h->grid_sweep + h->grid_reduce) : 0) +
                    h->npairs * 36 + 16 * h->ngroups + 8LL * (long long)ct.head_node.size();
   if (h->max_device_bytes > 0 && need > h->max_device_bytes) return BDD_ENOMEM;
 
@@ -821,6 +827,12 @@ int setup_device(bdd_solver *h, const Layout &L, const float *c, const CutTables
     h->d_lohi = reinterpret_cast<int2 *>(tmp);
   }
   if (h->lanes2) RC(upload(h, &h->d_lane_code, L.lane_code));
+  if (!L.node_rec.empty()) {
+    unsigned *tmp = nullptr;
+    RC(upload(h, &tmp, L.node_rec));
+    h->d_node_rec = reinterpret_cast<uint2 *>(tmp);
+    h->rec0 = (int)L.rec0;
+  }
   RC(h->alloc(&h->d_fm, N));
   RC(h->alloc(&h->d_bm, N));
   RC(h->alloc(&h->d_lam, O));
@@ -1049,6 +1061,22 @@ HostBDDs probe_instance(const HostBDDs &H, const std::vector<unsigned char> &key
   return P;
 }
 
+// Teams of 16 and 32 lanes push a forward layer with three shuffles per lane of the team, some 1300 and
+// 2500 cycles; a block tile takes about 450 whatever its width up to 128, but four warps per BDD
+// where a team has half of one or one.  With at most kFewWide such BDDs (four blocks per SM) there is
+// room for that and the chain decides: they go to block tiles (64x64 tomography in pieces of 32
+// layers, 300 of them: forward sweep 38 us with teams).  A smoothed team's forward layer is a chain of
+// up to 32 or 64 soft minima where a block tile's has one per predecessor; the sums and soft minima
+// run in the same order either way (lanes without a node add nothing), so the bits are the same.
+constexpr long long kFewWide = 608;
+void few_wide(bdd_solver *h, const HostBDDs &H, const std::vector<unsigned char> &keys) {
+  long long count = 0;
+  for (long long b = 0; b < H.nb(); ++b) count += keys[b] / kDepthBuckets >= 4 && keys[b] / kDepthBuckets < kWarpClasses;
+  if (count == 0 || count > kFewWide) return;
+  for (int k = 4 * kDepthBuckets; k < kWarpClasses * kDepthBuckets; ++k)
+    if (h->key_nodes[k] > 0) h->key_class[k] = kWarpClasses;
+}
+
 // ms of one forward plus one backward update sweep of the probe in the given layout (-1: failed)
 float probe_time(const HostBDDs &P, bool lanes2, const int *class_of_key) {
   bdd_solver *h = new (std::nothrow) bdd_solver();
@@ -1111,14 +1139,14 @@ float probe_time(const HostBDDs &P, bool lanes2, const int *class_of_key) {
 // Chooses the tile class of every key of a plain solver's BDDs (see above).  allow_lanes: lane
 // tiles are a candidate for widths <= 2 (-1 tuned, 0 never, 1 always).  Fills h->key_*, sets
 // h->lanes2; returns a BDD_* status.
-int tune_layout(bdd_solver *h, const HostBDDs &H, int allow_lanes) {
-  const std::vector<unsigned char> keys = bdd_keys(H, h->key_nodes);
+int tune_layout(bdd_solver *h, const HostBDDs &H, const std::vector<unsigned char> &keys, int allow_lanes) {
   const long long min_nodes = std::max(kProbeMin, H.N() / 100);
   bool any_lane = false;
   for (int k = 0; k < kLayoutKeys; ++k) {
     if (h->key_nodes[k] == 0) continue;
     const int wc = k / kDepthBuckets;
     if (wc == kWarpClasses) continue;  // block tiles: no alternative
+    if (h->key_class[k] == kWarpClasses) continue;  // settled (few_wide)
     // candidates: [default, alternative]; for widths <= 2 the teams of two lanes (class 1) and
     // the lane tiles (class 0 with lanes2)
     const bool narrow = wc <= 1;
@@ -1485,7 +1513,11 @@ int bdd_build(int n, int m, const long long *row_ptr, const int *col, const int 
     DeviceGuard dg(opt.device);
     rc = dg.ok ? BDD_OK : BDD_ECUDA;
     try {
-      if (rc == BDD_OK) rc = tune_layout(h, H, opt.lanes);
+      if (rc == BDD_OK) {
+        const std::vector<unsigned char> keys = bdd_keys(H, h->key_nodes);
+        few_wide(h, H, keys);
+        rc = tune_layout(h, H, keys, opt.lanes);
+      }
     } catch (const std::bad_alloc &) {
       rc = BDD_ENOMEM;
     }
@@ -1495,7 +1527,11 @@ int bdd_build(int n, int m, const long long *row_ptr, const int *col, const int 
     }
     keyed = true;
   } else {
-    bdd_keys(H, h->key_nodes);
+    const std::vector<unsigned char> keys = bdd_keys(H, h->key_nodes);
+    if (h->schedule == 1 && opt.tune_layout != 0) {
+      few_wide(h, H, keys);
+      keyed = true;  // (the other keys keep their defaults)
+    }
   }
   Layout L;
   try {

@@ -146,4 +146,26 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// The predecessors of a node in node order, a node's 0-arc before its 1-arc, from its record (the
+// second word of SweepParams::node_rec; W: the place that stands for none).
+struct PredRuns {
+  int i, ie, j, je;  // next and end of those by 0-arcs and by 1-arcs
+  __device__ __forceinline__ PredRuns(unsigned rec, int W) {
+    const unsigned q0 = rec & 0xffffu, q1 = rec >> 16;
+    i = (int)(q0 & 1023u);
+    ie = i == W ? i : i + (int)(q0 >> 10) + 1;
+    j = (int)(q1 & 1023u);
+    je = j == W ? j : j + (int)(q1 >> 10) + 1;
+  }
+  __device__ __forceinline__ bool more() const { return i < ie || j < je; }
+  __device__ __forceinline__ bool zero() const { return j >= je || (i < ie && i <= j); }
+  __device__ __forceinline__ int node() const { return zero() ? i : j; }
+  __device__ __forceinline__ bool take() {  // whether it was a 1-arc
+    const bool z = zero();
+    if (z) ++i;
+    else ++j;
+    return !z;
+  }
+};
+
 }  // namespace bdd

@@ -121,6 +121,8 @@ constexpr int kPersistWarps = kPersistThreads / 32;
 constexpr int kSubBlocks = kPersistThreads / kBlockThreads;
 constexpr int kMaxBlockTileWidth = 12288;           // two float layer buffers in shared memory
 constexpr int kMaxBlockTileDepth = 8192;
+constexpr int kFastWidth = 512;                     // widest layer of the one-barrier block tiles
+constexpr int kFastPreds = 63;                      // most predecessors of a node by one kind of arc there
 
 // Shared-memory stage of one warp: a window of kWinLayers layers of a warp tile (at most 32
 // occurrences and 32 nodes per layer), plus the node offsets and backward messages of the layer
@@ -214,6 +216,8 @@ struct Layout {
   hvec<int> var_occ;            // [O] device occurrence of each slot
   hvec<unsigned char> slot_dir; // [O] kDirForward / kDirBackward bits of each slot
   hvec<int> occ_of_canon;       // canonical occurrence -> device occurrence
+  hvec<unsigned> node_rec;      // [2 nodes of block tiles] see SweepParams::node_rec; empty: not used
+  long long rec0 = 0;           // first node of the block tiles
 };
 
 // Keys of the layout tuner: a BDD's natural class (the smallest team of 2^c >= its widest
@@ -426,6 +430,11 @@ struct SweepParams {
   float omega;
   float alpha;          // smoothing temperature (0: min-sum)
   float inv_alpha;
+  // one-barrier block tiles: a record per node from node rec0 on, {0-arc | 1-arc << 16 as places in the
+  // next layer's row (block_buf: bot, block_buf + 1: top), predecessors by 0-arcs | by 1-arcs << 16,
+  // each the first one's place | (their number - 1) << 10 (block_buf: none)}; null: the general form
+  const uint2 *node_rec;
+  int rec0;
   const float *copy_val; // sub-BDDs: mu_bar of every copy-arc pair (backward message of kCopy0 - k)
   int split;             // sub-BDDs: layer-0 forward messages are the root messages held in fm, and
                          // E^j is the minimum over the first layer of fm + bm
@@ -556,7 +565,7 @@ int cut_roots_launch(const CutParams &c, cudaStream_t stream);
 
 // Launch wrappers (kernels.cu).  All enqueue on `stream` and return 0 or -5 (launch failure).
 size_t sweep_smem_bytes(int block_buf, int block_depth_buf, int staging = 0, bool lanes2 = false,
-                        bool smooth = false);
+                        bool smooth = false, bool fast = false);
 size_t sweep_warp_smem(int staging, bool lanes2);
 int sweep_resident_blocks(size_t smem, int *blocks);  // blocks of a sweep launch per SM
 size_t persist_smem_bytes(int block_buf, int block_depth_buf);

@@ -21,6 +21,8 @@
 // barriers per iteration.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "internal.h"
 #include "device_common.cuh"
 
@@ -1546,9 +1548,18 @@ __device__ __forceinline__ int2 narrow_arcs(const SweepParams &p, const int *off
   return gt < off[l + 1] - node0 ? p.lohi[node0 + gt] : make_int2(kNone, kNone);
 }
 
-// SMOOTH: the forward step pulls instead of pushing -- node v of layer l + 1 aggregates its
-// in-arcs scanning the nodes of layer l in order, 0-arc before 1-arc (the soft minimum is not
-// associative in floating point, so a fixed order replaces the atomic minimum)
+// the predecessors of this thread's node in layer l (second word of its record)
+__device__ __forceinline__ unsigned narrow_pred(const SweepParams &p, const int *off, int l, int depth, int gt) {
+  const unsigned none = (unsigned)p.block_buf | (unsigned)p.block_buf << 16;
+  if (l >= depth || !p.node_rec) return none;
+  const int node0 = off[l];
+  return gt < off[l + 1] - node0 ? p.node_rec[BDD_NODE(p, node0 + gt) - p.rec0].y : none;
+}
+
+// SMOOTH: the forward step pulls instead of pushing -- node v of layer l + 1 aggregates its in-arcs
+// in the order of the nodes of layer l, 0-arc before 1-arc (the soft minimum is not associative in
+// floating point, so a fixed order replaces the atomic minimum).  Its predecessors come with its
+// record, loaded two layers ahead; without records it scans the layer.
 template <int MODE, bool SPLIT, bool SMOOTH = false>
 __device__ __forceinline__ void block_forward_narrow(const SweepParams &p, const Phase &ph, int tile,
                                                      const GroupSmem &g, int group, int gt, double &bacc) {
@@ -1564,6 +1575,8 @@ __device__ __forceinline__ void block_forward_narrow(const SweepParams &p, const
     if (gt < off[1] - n0) cur[gt] = SPLIT ? p.fm[n0 + gt] : 0.f;
   }
   int2 lh = narrow_arcs(p, off, 0, depth, gt), lh1 = narrow_arcs(p, off, 1, depth, gt);
+  unsigned pred1 = SMOOTH ? narrow_pred(p, off, 1, depth, gt) : 0u;
+  int slot = is_update(MODE) && gt == 0 ? p.occ_slot[occ0] : 0;
   float t0 = 0.f, t1 = 0.f;
   if (is_update(MODE)) {
     t0 = target_bm<SPLIT>(p.bm, p.copy_val, lh.x);
@@ -1578,12 +1591,14 @@ __device__ __forceinline__ void block_forward_narrow(const SweepParams &p, const
       u1 = target_bm<SPLIT>(p.bm, p.copy_val, lh1.y);
     }
     const int2 lh2 = narrow_arcs(p, off, l + 2, depth, gt);
+    const unsigned pred2 = SMOOTH ? narrow_pred(p, off, l + 2, depth, gt) : 0u;
+    const int slot1 = is_update(MODE) && gt == 0 && l + 1 < depth ? p.occ_slot[occ0 + l + 1] : 0;
     const int o = occ0 + l;
     const int node0 = off[l], w = off[l + 1] - node0;
     const bool has = gt < w;
     const float f = has ? cur[gt] : inf();
     if (has) p.fm[BDD_NODE(p, node0 + gt)] = f;
-    if (SMOOTH && gt < p.block_buf) g.arcs[gt] = lh;  // read by the pull after the next barrier
+    if (SMOOTH && !p.node_rec && gt < p.block_buf) g.arcs[gt] = lh;  // read by the pull after the next barrier
     float lam = g.shr[l];
     const bool more = l + 1 < depth;
     // nxt was last read before the previous layer's final barrier
@@ -1594,7 +1609,7 @@ __device__ __forceinline__ void block_forward_narrow(const SweepParams &p, const
       lam -= dd;
       if (gt == 0) {
         p.lam[BDD_OCC(p, o)] = lam;
-        ph.delta[BDD_OCC(p, p.occ_slot[o])] = dd;
+        ph.delta[BDD_OCC(p, slot)] = dd;
       }
     } else if (more) {
       group_sync(group);  // the resets of nxt before the pushes
@@ -1605,10 +1620,18 @@ __device__ __forceinline__ void block_forward_narrow(const SweepParams &p, const
         if (gt < off[l + 2] - next0) {
           const int v = next0 + gt;
           float acc = inf();
-          for (int u = 0; u < w; ++u) {
-            const int2 a = g.arcs[u];
-            if (a.x == v) acc = soft_min(acc, cur[u], p.alpha, p.inv_alpha);
-            if (a.y == v) acc = soft_min(acc, cur[u] + lam, p.alpha, p.inv_alpha);
+          if (p.node_rec) {
+            PredRuns r(pred1, p.block_buf);
+            while (r.more()) {
+              const float m = cur[r.node()];
+              acc = soft_min(acc, r.take() ? m + lam : m, p.alpha, p.inv_alpha);
+            }
+          } else {
+            for (int u = 0; u < w; ++u) {
+              const int2 a = g.arcs[u];
+              if (a.x == v) acc = soft_min(acc, cur[u], p.alpha, p.inv_alpha);
+              if (a.y == v) acc = soft_min(acc, cur[u] + lam, p.alpha, p.inv_alpha);
+            }
           }
           nxt[gt] = acc;
         }
@@ -1623,6 +1646,8 @@ __device__ __forceinline__ void block_forward_narrow(const SweepParams &p, const
     }
     lh = lh1;
     lh1 = lh2;
+    pred1 = pred2;
+    slot = slot1;
     t0 = u0;
     t1 = u1;
   }
@@ -1648,9 +1673,11 @@ __device__ __forceinline__ void block_backward_narrow(const SweepParams &p, cons
   int2 lh = narrow_arcs(p, off, last, depth, gt), lh1 = last >= 1 ? narrow_arcs(p, off, last - 1, depth, gt)
                                                                     : make_int2(kNone, kNone);
   float f = node_fm(last), f1 = node_fm(last - 1);
+  int slot = is_update(MODE) && gt == 0 ? p.occ_slot[occ0 + last] : 0;
   for (int l = last; l >= 0; --l) {
     const int2 lh2 = l >= 2 ? narrow_arcs(p, off, l - 2, depth, gt) : make_int2(kNone, kNone);
     const float f2 = node_fm(l - 2);
+    const int slot1 = is_update(MODE) && gt == 0 && l > 0 ? p.occ_slot[occ0 + l - 1] : 0;
     const int o = occ0 + l;
     const int node0 = off[l], w = off[l + 1] - node0, next0 = off[l + 1];
     const bool has = gt < w;
@@ -1664,7 +1691,7 @@ __device__ __forceinline__ void block_backward_narrow(const SweepParams &p, cons
         lam -= dd;
         if (gt == 0) {
           p.lam[BDD_OCC(p, o)] = lam;
-          ph.delta[BDD_OCC(p, p.occ_slot[o])] = dd;
+          ph.delta[BDD_OCC(p, slot)] = dd;
         }
       } else if (gt == 0 && p.out_m0) {
         const long long c = p.occ_csr[o];
@@ -1698,6 +1725,393 @@ __device__ __forceinline__ void block_backward_narrow(const SweepParams &p, cons
     lh1 = lh2;
     f = f1;
     f1 = f2;
+    slot = slot1;
+  }
+}
+
+// ---------------------------------------------------------------------------------------
+// block tiles of min-sum solvers whose layers have at most kFastWidth nodes: K nodes per thread, one
+// barrier per layer.
+//
+// A layer's chain is: the min-marginals of its nodes, their minimum over the block, the new
+// multiplier, the next layer's messages.  The messages cross threads (a node's neighbours belong
+// to others), and so does the minimum; both go through the same barrier:
+//   forward: every thread publishes its forward message before the barrier and, after it, pulls the
+//     next layer's from the predecessors (kept per node: in a reduced BDD the nodes whose 0-arc enters
+//     a node follow one another, and so do those whose 1-arc does).  min over the 1-arcs of
+//     (f + lambda) is (min f) + lambda: rounding is monotone, so these are the bits of the pushes.
+//   backward: every thread publishes the messages of its two arc targets before the barrier; after
+//     it everyone knows the multiplier and forms a neighbour's new message min(b0, lambda + b1)
+//     itself.
+// A node's record (SweepParams::node_rec) holds its arcs as places in the next layer's row, with two
+// places behind the row for bot and top, and its predecessors, a place for none: after the barrier
+// a thread reads everything it needs at once, without a branch.  Records and the other direction's
+// messages of the next R - 1 layers are under way as cp.async copies; offsets, multipliers and slots
+// are staged once, multipliers and differences written back after the last layer, so no layer
+// waits on global memory.
+//
+// Bound by the chain of instructions: rows of up to 300 variables (154 tiles, 300 layers, up to 151 nodes)
+// take 109 us a forward and 85 us a backward sweep, 0.36 and 0.28 us a layer (165 warp instructions a
+// layer at 4.3 cycles), where the plain form -- three barriers, atomic minima, arc targets fetched one
+// layer ahead -- took 348 and 227 us; 64x64 tomography 41 and 43 us against 74 and 61.
+// ---------------------------------------------------------------------------------------
+__host__ __device__ constexpr int fast_ring(int K) { return K < 4 ? 8 : 5; }
+__host__ __device__ constexpr int fast_k(int W) { return W <= kBlockThreads ? 1 : W <= 2 * kBlockThreads ? 2 : 4; }
+
+struct FastSmem {
+  float2 *red;   // [2][kWarpsPerBlock] the warps' minima of a layer
+  float2 *rows;  // [2][W + 4] published messages; place W: bot, W + 1: top
+  char *ring;    // [R] slots of a layer: records [W], messages [W + 4] (same places behind)
+  float *lam;    // [depth] multipliers (with the shares the sweep adds), later the new ones
+  float *diff;   // [depth] differences (folded pass: see fast_backward)
+  int *slot;     // [depth]
+  int *off;      // [depth + 4] node offsets, the last one repeated
+  int W;
+};
+__host__ __device__ __forceinline__ int fast_slot_bytes(int W) { return 12 * W + 16; }
+__host__ __device__ __forceinline__ size_t fast_bytes(int W, int depth) {
+  return 2 * kWarpsPerBlock * sizeof(float2) + 2 * (size_t)(W + 4) * sizeof(float2) +
+         (size_t)fast_ring(fast_k(W)) * fast_slot_bytes(W) + 16 * (size_t)depth + 16;
+}
+__device__ __forceinline__ FastSmem fast_smem(float *base, const SweepParams &p) {
+  FastSmem s;
+  s.W = p.block_buf;  // a multiple of 4
+  s.red = reinterpret_cast<float2 *>(base);
+  s.rows = s.red + 2 * kWarpsPerBlock;
+  s.ring = reinterpret_cast<char *>(s.rows + 2 * (s.W + 4));
+  s.lam = reinterpret_cast<float *>(s.ring + (size_t)fast_ring(fast_k(s.W)) * fast_slot_bytes(s.W));
+  s.diff = s.lam + p.block_depth_buf;
+  s.slot = reinterpret_cast<int *>(s.diff + p.block_depth_buf);
+  s.off = s.slot + p.block_depth_buf;
+  return s;
+}
+
+__device__ __forceinline__ float warp_min(float v) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+
+// the block's minima of a layer from the warps'
+__device__ __forceinline__ float2 fast_minima(const float2 *red) {
+  const float4 a = *reinterpret_cast<const float4 *>(red), b = *reinterpret_cast<const float4 *>(red + 2);
+  static_assert(kWarpsPerBlock == 4, "two float4 hold the warps' minima");
+  return make_float2(fminf(fminf(a.x, a.z), fminf(b.x, b.z)), fminf(fminf(a.y, a.w), fminf(b.y, b.w)));
+}
+
+template <int MODE>
+__device__ __forceinline__ void fast_stage(const SweepParams &p, const FastSmem &s, int occ0, int depth, int gt) {
+  for (int l = gt; l <= depth + 3; l += kBlockThreads) s.off[l] = p.occ_node_off[occ0 + min(l, depth)];
+  for (int l = gt; l < depth; l += kBlockThreads) {
+    s.lam[l] = p.lam[occ0 + l] + (MODE != kMessages ? p.share_occ[occ0 + l] : 0.f);
+    if (is_update(MODE)) s.slot[l] = p.occ_slot[occ0 + l];
+  }
+  // what lies behind the rows: +inf for bot (and no predecessor), 0 for top
+  if (gt < 2) {
+    s.rows[gt * (s.W + 4) + s.W] = make_float2(inf(), inf());
+    s.rows[gt * (s.W + 4) + s.W + 1] = make_float2(0.f, inf());
+  }
+  if (gt < fast_ring(fast_k(s.W))) {
+    float *m = reinterpret_cast<float *>(s.ring + (size_t)gt * fast_slot_bytes(s.W) + 8 * s.W);
+    m[s.W] = inf();
+    m[s.W + 1] = 0.f;
+  }
+  group_sync(0);
+}
+// new multipliers and differences of an update sweep
+__device__ __forceinline__ void fast_write(const SweepParams &p, const Phase &ph, const FastSmem &s, int occ0, int depth,
+                                           int gt) {
+  group_sync(0);
+  for (int l = gt; l < depth; l += kBlockThreads) {
+    p.lam[BDD_OCC(p, occ0 + l)] = s.lam[l];
+    ph.delta[BDD_OCC(p, s.slot[l])] = s.diff[l];
+  }
+}
+
+// Copies of one layer (nodes [n0, n0 + w)) into a ring slot: records and, if wanted, messages.
+template <int K>
+__device__ __forceinline__ void fast_issue(const SweepParams &p, char *slot, int W, const float *msgs, int n0, int w, int gt) {
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const int t = gt + k * kBlockThreads;
+    if (t < w) {
+      cp_async8(slot + 8 * t, p.node_rec + (BDD_NODE(p, n0 + t) - p.rec0));
+      if (msgs) cp_async4(slot + 8 * W + 4 * t, msgs + BDD_NODE(p, n0 + t));
+    }
+  }
+}
+
+template <int MODE, bool SPLIT, int K>
+__device__ __forceinline__ void fast_forward(const SweepParams &p, const Phase &ph, int tile, const FastSmem &s, int gt) {
+  constexpr int R = fast_ring(K);
+  const int W = s.W, SB = fast_slot_bytes(W), lane = gt & 31, warp = gt >> 5;
+  const int occ0 = p.tile_occ0[tile], depth = p.bdd_depth[p.tile_bdd0[tile]];
+  const int *off = s.off;
+  fast_stage<MODE>(p, s, occ0, depth, gt);
+  const float *msgs = is_update(MODE) ? p.bm : nullptr;
+#pragma unroll
+  for (int l = 0; l < R - 1; ++l) {
+    if (l < depth) fast_issue<K>(p, s.ring + l * SB, W, msgs, off[l], off[l + 1] - off[l], gt);
+    cp_async_commit();
+  }
+  const uint2 none = make_uint2((unsigned)W | (unsigned)W << 16, (unsigned)W | (unsigned)W << 16);
+  auto record = [&](const char *slot, int w, int k) {
+    const int t = gt + k * kBlockThreads;
+    return t < w ? reinterpret_cast<const uint2 *>(slot)[t] : none;
+  };
+  float f[K], t0[K], t1[K];
+  uint2 rec[K];  // of the next layer
+  cp_async_wait_group<R - 4>();  // layers 0 .. 2
+  group_sync(0);
+#pragma unroll
+  for (int k = 0; k < K; ++k) {  // the root, or a piece's roots with their root messages (sub-BDDs)
+    const int t = gt + k * kBlockThreads, w = off[1] - off[0];
+    f[k] = t < w ? (SPLIT ? p.fm[off[0] + t] : 0.f) : inf();
+    const uint2 r = record(s.ring, w, k);
+    const float *m = reinterpret_cast<const float *>(s.ring + SB + 8 * W);
+    t0[k] = t1[k] = inf();
+    if (is_update(MODE)) {
+      t0[k] = m[r.x & 0xffffu];
+      t1[k] = m[r.x >> 16];
+    }
+    rec[k] = record(s.ring + SB, off[2] - off[1], k);
+  }
+  // sub-BDDs: an arc across a cut has its message in the copy-arc duals (the last layer only)
+  auto cut_targets = [&](int n0, int w) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int t = gt + k * kBlockThreads;
+      if (t < w) {
+        const int2 a = p.lohi[BDD_NODE(p, n0 + t)];
+        t0[k] = terminal_bm<SPLIT>(p.copy_val, a.x);
+        t1[k] = terminal_bm<SPLIT>(p.copy_val, a.y);
+      }
+    }
+  };
+  if (SPLIT && is_update(MODE) && depth == 1) cut_targets(off[0], off[1] - off[0]);
+  int n0 = off[0], n1 = off[1], n2 = off[2];
+  float lam = s.lam[0];
+  // slots of layers l + 2 (its messages and records are read after this layer's barrier) and l + R - 1
+  const char *ahead = s.ring + 2 * SB;
+  char *fill = s.ring + (R - 1) * SB;
+  const char *const ring_end = s.ring + R * SB;
+  for (int l = 0; l < depth; ++l) {
+    float2 *rows = s.rows + (l & 1) * (W + 4);
+    float2 *red = s.red + (l & 1) * kWarpsPerBlock;
+    float a0 = inf(), a1 = inf();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int t = gt + k * kBlockThreads;
+      if (is_update(MODE)) {
+        a0 = fminf(a0, f[k] + t0[k]);
+        a1 = fminf(a1, f[k] + lam + t1[k]);
+      }
+      if (t < n1 - n0) {
+        rows[t].x = f[k];
+        p.fm[BDD_NODE(p, n0 + t)] = f[k];
+      }
+    }
+    if (is_update(MODE)) {
+      a0 = warp_min(a0);
+      a1 = warp_min(a1);
+      if (lane == 0) red[warp] = make_float2(a0, a1);
+    }
+    cp_async_wait_group<R - 4>();  // this thread's part of layer l + 2
+    group_sync(0);
+    const int n3 = off[l + 3 < depth ? l + 3 : depth];
+    const float lam_next = s.lam[l + 1 < depth ? l + 1 : l];
+    float from0[K], from1[K];  // least messages over the 0- and the 1-arcs into this thread's next nodes
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const unsigned q0 = rec[k].y & 0xffffu, q1 = rec[k].y >> 16;  // place | (predecessors - 1) << 10
+      from0[k] = rows[q0 & 1023u].x;
+      from1[k] = rows[q1 & 1023u].x;
+      if ((q0 | q1) >> 10) {  // nodes merged from several of the layer before
+        for (unsigned j = 1; j <= q0 >> 10; ++j) from0[k] = fminf(from0[k], rows[(q0 & 1023u) + j].x);
+        for (unsigned j = 1; j <= q1 >> 10; ++j) from1[k] = fminf(from1[k], rows[(q1 & 1023u) + j].x);
+      }
+      if (is_update(MODE)) {
+        const float *m = reinterpret_cast<const float *>(ahead + 8 * W);
+        t0[k] = m[rec[k].x & 0xffffu];
+        t1[k] = m[rec[k].x >> 16];
+      }
+      rec[k] = record(ahead, n3 - n2, k);
+    }
+    float la = lam;
+    if (is_update(MODE)) {
+      const float2 m = fast_minima(red);
+      const float dd = p.omega * mm_difference(m.x, m.y);
+      la -= dd;
+      if (gt == 0) {
+        s.lam[l] = la;
+        s.diff[l] = dd;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) f[k] = fminf(from0[k], from1[k] + la);
+    if (SPLIT && is_update(MODE) && l + 2 == depth) cut_targets(n1, n2 - n1);
+    if (l + R - 1 < depth) fast_issue<K>(p, fill, W, msgs, off[l + R - 1], off[l + R] - off[l + R - 1], gt);
+    cp_async_commit();
+    fill = fill + SB == ring_end ? s.ring : fill + SB;
+    ahead = ahead + SB == ring_end ? s.ring : ahead + SB;
+    lam = lam_next;
+    n0 = n1;
+    n1 = n2;
+    n2 = n3;
+  }
+  if (is_update(MODE)) fast_write(p, ph, s, occ0, depth, gt);
+}
+
+template <int MODE, bool SPLIT, int K>
+__device__ __forceinline__ void fast_backward(const SweepParams &p, const Phase &ph, int tile, const FastSmem &s, int gt) {
+  constexpr int R = fast_ring(K);
+  const int W = s.W, SB = fast_slot_bytes(W), lane = gt & 31, warp = gt >> 5;
+  const int bdd = p.tile_bdd0[tile], occ0 = p.tile_occ0[tile], depth = p.bdd_depth[bdd];
+  const int *off = s.off;
+  fast_stage<MODE>(p, s, occ0, depth, gt);
+  // (a thread reads only its own entries of the ring: no barrier is needed for them)
+#pragma unroll
+  for (int j = 0; j < R - 1; ++j) {
+    const int l = depth - 1 - j;
+    if (l >= 0) fast_issue<K>(p, s.ring + j * SB, W, p.fm, off[l], off[l + 1] - off[l], gt);
+    cp_async_commit();
+  }
+  float f[K], b0[K], b1[K], f_next[K];
+  unsigned arcs[K];  // of the next layer up
+  auto entry = [&](const char *slot, int w, int k, float &fv) {
+    const int t = gt + k * kBlockThreads;
+    fv = t < w ? reinterpret_cast<const float *>(slot + 8 * W)[t] : inf();
+    return t < w ? reinterpret_cast<const uint2 *>(slot)[t].x : (unsigned)W | (unsigned)W << 16;
+  };
+  cp_async_wait_group<R - 3>();  // layers depth - 1 and depth - 2
+  int n0 = off[depth - 1], n1 = off[depth];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const unsigned a = entry(s.ring, n1 - n0, k, f[k]);
+    if (SPLIT) {  // a piece's last arcs may cross a cut
+      const int t = gt + k * kBlockThreads;
+      b0[k] = b1[k] = inf();
+      if (t < n1 - n0) {
+        const int2 q = p.lohi[BDD_NODE(p, n0 + t)];
+        b0[k] = terminal_bm<SPLIT>(p.copy_val, q.x);
+        b1[k] = terminal_bm<SPLIT>(p.copy_val, q.y);
+      }
+    } else {  // bot or top, behind the rows
+      b0[k] = s.rows[a & 0xffffu].x;
+      b1[k] = s.rows[a >> 16].x;
+    }
+    f_next[k] = inf();
+    arcs[k] = (unsigned)W | (unsigned)W << 16;
+    if (depth > 1) arcs[k] = entry(s.ring + SB, n0 - off[depth - 2], k, f_next[k]);
+  }
+  const char *ahead = s.ring + 2 * SB;  // slots of layers l - 2 and l - (R - 1)
+  char *fill = s.ring + (R - 1) * SB;
+  const char *const ring_end = s.ring + R * SB;
+  float lam = s.lam[depth - 1];
+  for (int l = depth - 1; l >= 0; --l) {
+    float2 *rows = s.rows + (l & 1) * (W + 4);
+    float2 *red = s.red + (l & 1) * kWarpsPerBlock;
+    float a0 = inf(), a1 = inf();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int t = gt + k * kBlockThreads;
+      if (MODE != kMessages) {
+        a0 = fminf(a0, f[k] + b0[k]);
+        a1 = fminf(a1, f[k] + lam + b1[k]);
+      }
+      if (t < n1 - n0) rows[t] = make_float2(b0[k], b1[k]);
+    }
+    if (MODE != kMessages) {
+      a0 = warp_min(a0);
+      a1 = warp_min(a1);
+      if (lane == 0) red[warp] = make_float2(a0, a1);
+    }
+    cp_async_wait_group<R - 4>();  // layer l - 2
+    group_sync(0);
+    float2 q0[K], q1[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      q0[k] = rows[arcs[k] & 0xffffu];
+      q1[k] = rows[arcs[k] >> 16];
+    }
+    const float lam_next = s.lam[l > 0 ? l - 1 : 0];
+    const int np = l > 0 ? off[l - 1] : n0, npp = l > 1 ? off[l - 2] : np;
+    float la = lam;
+    if (MODE != kMessages) {
+      const float2 m = fast_minima(red);
+      if (is_update(MODE)) {
+        const float dd = p.omega * mm_difference(m.x, m.y);
+        la -= dd;
+        if (gt == 0) {
+          s.lam[l] = la;
+          s.diff[l] = dd;
+        }
+      } else if (gt == 0) {  // the layer's difference and slot are not needed
+        s.diff[l] = m.x;
+        s.slot[l] = __float_as_int(m.y);
+      }
+    }
+    // Alg. 3: m_bwd(v) = min(m_bwd(v0) + 0, m_bwd(v1) + lambda)
+    float e = inf();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int t = gt + k * kBlockThreads;
+      const float bcur = fminf(b0[k], la + b1[k]);
+      if (t < n1 - n0) {
+        p.bm[BDD_NODE(p, n0 + t)] = bcur;
+        if (SPLIT) e = fminf(e, f[k] + bcur);
+        else if (t == 0) e = bcur;
+      }
+      b0[k] = fminf(q0[k].x, la + q0[k].y);
+      b1[k] = fminf(q1[k].x, la + q1[k].y);
+      f[k] = f_next[k];
+      arcs[k] = entry(ahead, np - npp, k, f_next[k]);
+    }
+    if (l == 0) {  // E^j at the root; a piece: min over its roots of fm + bm
+      if (SPLIT) {
+        e = warp_min(e);
+        float2 *last = s.red + kWarpsPerBlock;  // (layer 0 used the other half)
+        if (lane == 0) last[warp] = make_float2(e, e);
+        group_sync(0);
+        e = fast_minima(last).x;
+      }
+      if (gt == 0) p.bdd_E[BDD_BDD(p, bdd)] = e;
+    }
+    if (l - (R - 1) >= 0) fast_issue<K>(p, fill, W, p.fm, off[l - (R - 1)], off[l - (R - 2)] - off[l - (R - 1)], gt);
+    cp_async_commit();
+    fill = fill + SB == ring_end ? s.ring : fill + SB;
+    ahead = ahead + SB == ring_end ? s.ring : ahead + SB;
+    lam = lam_next;
+    n1 = n0;
+    n0 = np;
+  }
+  if (is_update(MODE)) fast_write(p, ph, s, occ0, depth, gt);
+  if (MODE == kFolded && p.out_m0) {
+    group_sync(0);
+    for (int l = gt; l < depth; l += kBlockThreads) {
+      const long long c = p.occ_csr[occ0 + l];
+      p.out_m0[BDD_CSR(p, c)] = s.diff[l];
+      p.out_m1[BDD_CSR(p, c)] = __int_as_float(s.slot[l]);
+    }
+  }
+}
+
+template <bool FWD, int MODE, bool SPLIT>
+__device__ __forceinline__ void fast_block(const SweepParams &p, const Phase &ph, int tile, float *smem, int gt) {
+  const FastSmem s = fast_smem(smem, p);
+  switch (fast_k(s.W)) {
+    case 1:
+      if (FWD) fast_forward<MODE, SPLIT, 1>(p, ph, tile, s, gt);
+      else fast_backward<MODE, SPLIT, 1>(p, ph, tile, s, gt);
+      break;
+    case 2:
+      if (FWD) fast_forward<MODE, SPLIT, 2>(p, ph, tile, s, gt);
+      else fast_backward<MODE, SPLIT, 2>(p, ph, tile, s, gt);
+      break;
+    default:
+      if (FWD) fast_forward<MODE, SPLIT, 4>(p, ph, tile, s, gt);
+      else fast_backward<MODE, SPLIT, 4>(p, ph, tile, s, gt);
+      break;
   }
 }
 
@@ -1858,12 +2272,14 @@ __global__ void __launch_bounds__(kBlockThreads) sweep_kernel(const SweepParams 
     if (tile >= p.class_tile_off[kWarpClasses + 1]) return;  // uniform across the block
     pdl_wait();
     const GroupSmem g = group_smem(smem, p);
-    if (p.block_buf <= kBlockThreads) {
+    if constexpr (SMOOTH) {
       if (FWD)
         block_forward_narrow<MODE, SPLIT, SMOOTH>(p, ph, tile, g, 0, threadIdx.x, bacc);
       else
         block_backward_narrow<MODE, SPLIT, SMOOTH>(p, ph, tile, g, 0, threadIdx.x, bacc);
-    } else if constexpr (!SMOOTH) {
+    } else if (p.node_rec) {
+      fast_block<FWD, MODE, SPLIT>(p, ph, tile, smem, threadIdx.x);
+    } else {
       if (FWD)
         block_forward<MODE, SPLIT>(p, ph, tile, g, 0, threadIdx.x, bacc);
       else
@@ -2275,17 +2691,20 @@ int sweep_resident_blocks(size_t smem, int *blocks) {
              : -5;
 }
 
-size_t sweep_smem_bytes(int block_buf, int block_depth_buf, int staging, bool lanes2, bool smooth) {
-  const size_t warp_part = kWarpsPerBlock * sweep_warp_smem(staging, lanes2);
-  const size_t group_part = group_floats(block_buf, block_depth_buf, smooth) * sizeof(float);
-  return warp_part > group_part ? warp_part : group_part;
+// shared memory of a block tile in a per-phase launch (fast: the one-barrier form)
+static size_t block_tile_bytes(int block_buf, int block_depth_buf, bool smooth, bool fast) {
+  if (!fast) return group_floats(block_buf, block_depth_buf, smooth) * sizeof(float);
+  return fast_bytes(block_buf, block_depth_buf);
+}
+
+size_t sweep_smem_bytes(int block_buf, int block_depth_buf, int staging, bool lanes2, bool smooth, bool fast) {
+  return std::max(kWarpsPerBlock * sweep_warp_smem(staging, lanes2),
+                  block_tile_bytes(block_buf, block_depth_buf, smooth, fast));
 }
 
 // the same for a layout whose warp tiles are all lane tiles (min-sum sweeps)
-size_t lane_only_smem_bytes(int block_buf, int block_depth_buf) {
-  const size_t warp_part = kWarpsPerBlock * kLaneSmemBytes;
-  const size_t group_part = group_floats(block_buf, block_depth_buf, false) * sizeof(float);
-  return warp_part > group_part ? warp_part : group_part;
+static size_t lane_only_smem_bytes(int block_buf, int block_depth_buf, bool fast) {
+  return std::max(kWarpsPerBlock * kLaneSmemBytes, block_tile_bytes(block_buf, block_depth_buf, false, fast));
 }
 
 size_t persist_smem_bytes(int block_buf, int block_depth_buf) {
@@ -2307,8 +2726,8 @@ int sweep_launch(bool forward, int mode, const SweepParams &p_in, int grid, cuda
   // more blocks fit on an SM
   const bool lane_only = p.lanes2 && p.class_tile_off[1] == p.class_tile_off[kWarpClasses];
   p.warp_smem = lane_only ? (int)kLaneSmemBytes : (int)sweep_warp_smem(staging, p.lanes2 != 0);
-  size_t smem = sweep_smem_bytes(p.block_buf, p.block_depth_buf, staging, p.lanes2 != 0, p.alpha > 0.f);
-  if (lane_only) smem = lane_only_smem_bytes(p.block_buf, p.block_depth_buf);
+  size_t smem = sweep_smem_bytes(p.block_buf, p.block_depth_buf, staging, p.lanes2 != 0, p.alpha > 0.f, p.node_rec && !(p.alpha > 0.f));
+  if (lane_only) smem = lane_only_smem_bytes(p.block_buf, p.block_depth_buf, p.node_rec != nullptr);
   int rc = 0;
   if (p.split) {  // sub-BDDs: min-sum only, no fused pending pass
     if (p.alpha > 0.f || mode == kUpdateFused) return -5;

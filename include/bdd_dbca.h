@@ -99,7 +99,8 @@ typedef struct {
                                  (default): plain solvers (alpha = 0, no split, averaging 0)
                                  whose layout is left to the library too (lanes != 0, staging and
                                  tune_layout not forced on, no layout_classes) and whose BDDs have
-                                 layers of at most two nodes and at most 32 of them run the
+                                 layers of at most four nodes and at most 32 of them (up to 128
+                                 layers of at most two nodes where few rows are so long) run the
                                  direct plan: every sweep forms the shares from the recorded
                                  differences itself and recomputes the messages it needs, two
                                  kernels per iteration; the others as 0.
@@ -287,7 +288,7 @@ int bdd_status_of_device_word(int word);
 
 /* Tile class of every layout key (see bdd_options.tune_layout), no counterpart in the paper:
  * nodes[k] nodes of the solver's BDDs with key k, cls[k] the class they run in (-1 none, 0..5
- * a team of 2^c lanes, 6 block tiles, 7 lane tiles), ms (NULL skips it) [2k], [2k + 1]: the
+ * a team of 2^c lanes, 6 block tiles, 7 lane tiles; in the direct plan also layers of four nodes), ms (NULL skips it) [2k], [2k + 1]: the
  * tuner's probe time of the default and the alternative class (-1: not probed).  Arrays of
  * BDD_LAYOUT_KEYS (2 BDD_LAYOUT_KEYS for ms), host. */
 int bdd_layout_table(const bdd_solver *h, long long *nodes, int *cls, float *ms);

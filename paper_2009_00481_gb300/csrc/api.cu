@@ -162,9 +162,10 @@ struct bdd_solver {
   bool direct = false;
   DirectLayout dlayout;          // kept in host memory for host_only == 2 only
   long long Od = 0, ext = 0;     // occurrences with padding, grouped values
-  int n_tiles = 0, deep_depth = 0, chains = 0, n_coop = 0, warp_depth = 0, heavy0 = 0, grid_direct = 0;
+  int n_tiles = 0, deep_depth = 0, chains = 0, n_coop = 0, warp_bytes = 0, occ4 = 0, heavy0 = 0, grid_direct = 0;
   size_t smem_direct = 0;
   int4 *d_tile = nullptr;
+  unsigned *d_code4 = nullptr;
   int *d_ref = nullptr, *d_home = nullptr, *d_heavy_of = nullptr;
   unsigned char *d_ext_deg = nullptr;
   float *d_diff_f = nullptr, *d_diff_b = nullptr;  // differences of the last forward / backward sweep
@@ -290,7 +291,9 @@ struct bdd_solver {
     p.deep_depth = deep_depth;
     p.chains = chains;
     p.n_coop = n_coop;
-    p.warp_depth = warp_depth;
+    p.warp_bytes = warp_bytes;
+    p.code4 = d_code4;
+    p.occ4 = occ4;
     p.omega = omega;
     p.bdd_E = d_bdd_E;
     p.partial = d_partial;
@@ -928,17 +931,24 @@ int setup_direct(bdd_solver *h, const DirectLayout &L, const float *c) {
   // layers, as long as there are at most as many as SMs (300x300 matching, 19 such tiles: a sweep of
   // 31 us with a warp to a tile, 16 with a block, 12.5 once the walks read a layer ahead); more of
   // them fill the GPU with a warp each
-  h->warp_depth = h->deep_depth;
+  int warp_depth = h->deep_depth;
+  h->n_coop = L.n_coop;
+  if (L.n_coop > 0) warp_depth = std::min(warp_depth, kLaneDeepDepth);
   if (h->deep_depth > kCoopDepth) {
     int coop = 0;
-    while (coop < L.n_tiles && (L.tile[4 * coop + 3] & kTileDepth) > kCoopDepth && (L.tile[4 * coop + 2] & kTileDeep)) ++coop;
-    const bool all = coop == L.n_tiles || (L.tile[4 * coop + 3] & kTileDepth) <= kCoopDepth;
+    while (coop < L.n_tiles && (L.tile[4 * coop + 3] & kTileDepth) > kCoopDepth && (L.tile[4 * coop + 2] & kTileDeep) &&
+           !(L.tile[4 * coop + 2] & kTileFour))
+      ++coop;
+    const bool all = coop == L.n_tiles || (L.tile[4 * coop + 2] & kTileFour) ||
+                     (L.tile[4 * coop + 3] & kTileDepth) <= kCoopDepth;
     if (coop <= nsm && all) {
       h->n_coop = coop;
-      h->warp_depth = std::min(h->deep_depth, kCoopDepth);
+      warp_depth = std::min(h->deep_depth, kCoopDepth);
     }
   }
-  h->smem_direct = (size_t)kLaneLayerBytes * std::max(kWarpsPerBlock * h->warp_depth, h->n_coop ? h->deep_depth : 0);
+  h->occ4 = (int)L.occ4;
+  h->warp_bytes = std::max(warp_depth * kLaneLayerBytes, L.four_depth * kLane4LayerBytes);
+  h->smem_direct = std::max((size_t)kWarpsPerBlock * h->warp_bytes, h->n_coop ? (size_t)h->deep_depth * kLaneLayerBytes : 0);
   if (h->smem_direct > 48 * 1024 && direct_set_smem(h->smem_direct)) return BDD_ECUDA;
   if (direct_resident_blocks(L.chains, h->smem_direct, &per_sm)) return BDD_ECUDA;
   // one wave of blocks at most: the warps take the tiles in turn (deepest first), so the bound has
@@ -946,7 +956,7 @@ int setup_direct(bdd_solver *h, const DirectLayout &L, const float *c) {
   const int wave = std::max(1, nsm) * std::max(1, per_sm);
   h->grid_direct = h->n_coop + std::max(1, std::min((L.n_tiles - h->n_coop + kWarpsPerBlock - 1) / kWarpsPerBlock, wave - h->n_coop));
   h->pdl_early = h->grid_direct < wave;
-  const long long need = 29 * Od + 12 * h->ext + 4 * (3 * n + 1) + 12 * nb + 16LL * L.n_tiles + 8LL * h->grid_direct + 1024 * 8;
+  const long long need = 29 * Od + 4LL * (long long)L.code4.size() + 12 * h->ext + 4 * (3 * n + 1) + 12 * nb + 16LL * L.n_tiles + 8LL * h->grid_direct + 1024 * 8;
   if (h->max_device_bytes > 0 && need > h->max_device_bytes) return BDD_ENOMEM;
   {
     int *tmp = nullptr;
@@ -958,6 +968,7 @@ int setup_direct(bdd_solver *h, const DirectLayout &L, const float *c) {
     h->n_heavy = (int)(L.heavy.size() / 4);
   }
   RC(upload(h, &h->d_lane_code, L.code));
+  RC(upload(h, &h->d_code4, L.code4));
   RC(upload(h, &h->d_ref, L.ref));
   RC(upload(h, &h->d_occ_csr, L.csr));
   RC(upload(h, &h->d_occ_var, L.var));
@@ -1210,6 +1221,10 @@ int export_direct(const bdd_solver *h, int *bdd_row, int *bdd_depth, int *occ_va
     read.code.resize(h->Od);
     read.var.resize(h->Od);
     read.csr.resize(h->Od);
+    read.occ4 = h->occ4;
+    read.code4.resize(h->Od - h->occ4);
+    if (h->Od > h->occ4)
+      CK(cudaMemcpy(read.code4.data(), h->d_code4, sizeof(unsigned) * (h->Od - h->occ4), cudaMemcpyDeviceToHost));
     CK(cudaEventSynchronize(h->ev_last));
     if (h->n_tiles) CK(cudaMemcpy(read.tile.data(), h->d_tile, sizeof(int4) * h->n_tiles, cudaMemcpyDeviceToHost));
     if (nb) CK(cudaMemcpy(read.bdd_depth.data(), h->d_bdd_depth, sizeof(int) * nb, cudaMemcpyDeviceToHost));
@@ -1222,7 +1237,7 @@ int export_direct(const bdd_solver *h, int *bdd_row, int *bdd_depth, int *occ_va
   std::vector<int> sorted_of_canon(nb), tile_of(nb, -1);
   for (long long s = 0; s < nb; ++s) sorted_of_canon[h->bdd_perm[s]] = (int)s;
   for (int t = 0; t < h->n_warp_tiles; ++t)
-    for (int q = 0; q < (L.tile[4 * t + 2] & (kTileDeep - 1)); ++q)
+    for (int q = 0; q < (L.tile[4 * t + 2] & kTileCount); ++q)
       if (L.tile[4 * t + 1] + q < nb) tile_of[L.tile[4 * t + 1] + q] = t;
   long long co = 0, cn = 0;
   for (long long cb = 0; cb < nb; ++cb) {
@@ -1235,17 +1250,22 @@ int export_direct(const bdd_solver *h, int *bdd_row, int *bdd_depth, int *occ_va
     for (int l = 0; l < depth; ++l, ++co) {
       const long long o = L.tile[4 * t] + 32LL * l + lane;
       if (co >= O) return BDD_EDEVICE;
-      const unsigned c = L.code[o];
-      const int w = (c >> 4) == (kDirectNoNode1 >> 4) ? 1 : 2;
+      const bool four = L.tile[4 * t + 2] & kTileFour;
+      const unsigned c = four ? L.code4[o - L.occ4] : L.code[o];
+      int w = (c >> 4) == (kDirectNoNode1 >> 4) ? 1 : 2;
+      if (four)
+        for (w = 1; w < 4 && ((c >> (6 * w)) & 63u) != kDirectNone4;) ++w;
+      const int bits = four ? 3 : 2;
+      const unsigned mask = four ? 7u : 3u, bot = four ? kDirectBot4 : kDirectBot;
       occ_var[co] = L.var[o];
       occ_csr[co] = L.csr[o];
       occ_width[co] = w;
       for (int q = 0; q < w; ++q, ++cn) {
         if (cn >= N) return BDD_EDEVICE;
-        const unsigned a0 = (c >> (4 * q)) & 3u, a1 = (c >> (4 * q + 2)) & 3u;
+        const unsigned a0 = (c >> (2 * bits * q)) & mask, a1 = (c >> (2 * bits * q + bits)) & mask;
         const int node0 = l + 1 == depth ? kTop : 0;
-        lo[cn] = a0 == 0 ? node0 : a0 == kDirectBot ? kBot : (int)a0;
-        hi[cn] = a1 == 0 ? node0 : a1 == kDirectBot ? kBot : (int)a1;
+        lo[cn] = a0 == 0 ? node0 : a0 == bot ? kBot : (int)a0;
+        hi[cn] = a1 == 0 ? node0 : a1 == bot ? kBot : (int)a1;
       }
     }
   }
@@ -1488,7 +1508,8 @@ int bdd_build(int n, int m, const long long *row_ptr, const int *col, const int 
     if (rc == BDD_OK) {
       h->lanes2 = L.class_tile_off[1] > 0;
       bdd_keys(H, h->key_nodes);
-      for (int k = 0; k < 2 * kDepthBuckets; ++k) h->key_class[k] = h->key_nodes[k] ? 0 : -1;
+      for (int k = 0; k < kLayoutKeys; ++k)  // lane tiles (bdd_layout_table)
+        h->key_class[k] = !h->key_nodes[k] ? -1 : k < 2 * kDepthBuckets ? 0 : kWarpClasses + 1;
       h->lane_O = h->O;
       h->lane_N = h->N;
       return finish_build(h, opt, c, out);

@@ -723,46 +723,60 @@ int build_layout(const HostBDDs &H, Layout *L, bool lanes2, const int *class_of_
 int build_direct_layout(const HostBDDs &H, DirectLayout *L, const int *var_deg) {
   const long long nb = H.nb(), O = H.O();
   const int n = H.n;
+  // two kinds of tiles: layers of at most two nodes, and of at most four (a layer never has more than
+  // twice the nodes of the one before, so a BDD of width 3 or 4 has at least three layers)
   std::atomic<bool> fits{true};
+  std::vector<unsigned char> four(nb);
   parallel_for(nb, 4096, [&](long long b0, long long b1) {
     for (long long b = b0; b < b1; ++b) {
       int w = 0;
       for (long long o = H.bdd_occ0[b]; o < H.bdd_occ0[b + 1]; ++o) w = std::max(w, H.occ_width[o]);
-      if (w > 2 || H.bdd_depth[b] > kLaneDeepDepth) fits.store(false);
+      four[b] = w > 2;
+      if (w > 4 || H.bdd_depth[b] > (w > 2 ? kLaneDeepDepth : kLaneCoopDepth)) fits.store(false);
     }
   });
   if (!fits.load()) return BDD_ETOOBIG;
-  // stable counting sort by depth, deepest first; ties keep ascending row order
+  // stable counting sort by kind and depth, deepest first; ties keep ascending row order
   const int D = H.max_depth;
-  std::vector<long long> cnt(D + 2, 0);
-  for (long long b = 0; b < nb; ++b) cnt[D - H.bdd_depth[b] + 1]++;
-  for (int t = 0; t <= D; ++t) cnt[t + 1] += cnt[t];
+  std::vector<long long> cnt(2 * (D + 1) + 1, 0);
+  auto key = [&](long long b) { return four[b] * (D + 1) + D - H.bdd_depth[b]; };
+  for (long long b = 0; b < nb; ++b) cnt[key(b) + 1]++;
+  for (int t = 0; t < 2 * (D + 1); ++t) cnt[t + 1] += cnt[t];
+  const long long n_two = cnt[D + 1];
   L->bdd_perm.resize(nb);
-  for (long long b = 0; b < nb; ++b) L->bdd_perm[cnt[D - H.bdd_depth[b]]++] = (int)b;
+  for (long long b = 0; b < nb; ++b) L->bdd_perm[cnt[key(b)]++] = (int)b;
   L->bdd_depth.resize(nb);
   parallel_for(nb, 1 << 14, [&](long long s0, long long s1) {
     for (long long t = s0; t < s1; ++t) L->bdd_depth[t] = H.bdd_depth[L->bdd_perm[t]];
   });
   // tiles of at most 32 BDDs, each a rectangle of its deepest BDD's depth; a depth that fills a tile
   // starts one of its own (a tile of one depth can be a chain tile)
-  std::vector<long long> run(D + 2, 0);  // BDDs of each depth
-  for (long long s = 0; s < nb; ++s) run[L->bdd_depth[s]]++;
   long long od = 0;
-  for (long long s = 0; s < nb;) {
-    const int depth = L->bdd_depth[s];
-    long long e = s + 1;
-    while (e < nb && e - s < 32 && (L->bdd_depth[e] == L->bdd_depth[e - 1] || run[L->bdd_depth[e]] < 32)) ++e;
-    const int t[4] = {(int)od, (int)s, (int)(e - s), depth};
-    L->tile.insert(L->tile.end(), t, t + 4);
-    od += 32LL * depth;
-    if (od > INT_MAX) return BDD_ETOOBIG;
-    s = e;
+  for (int kind = 0; kind < 2; ++kind) {
+    const long long end = kind ? nb : n_two;
+    std::vector<long long> run(D + 2, 0);  // BDDs of each depth
+    for (long long s = kind ? n_two : 0; s < end; ++s) run[L->bdd_depth[s]]++;
+    if (kind) L->occ4 = od;
+    for (long long s = kind ? n_two : 0; s < end;) {
+      const int depth = L->bdd_depth[s];
+      long long e = s + 1;
+      while (e < end && e - s < 32 && (L->bdd_depth[e] == L->bdd_depth[e - 1] || run[L->bdd_depth[e]] < 32)) ++e;
+      const int t[4] = {(int)od, (int)s, (int)(e - s) | (kind ? kTileFour | kTileDeep : 0), depth};
+      L->tile.insert(L->tile.end(), t, t + 4);
+      L->n_coop += depth > kLaneDeepDepth;
+      if (kind) L->four_depth = std::max(L->four_depth, depth);
+      od += 32LL * depth;
+      if (od > INT_MAX) return BDD_ETOOBIG;
+      s = e;
+    }
   }
+  if (L->n_coop > kCoopMost) return BDD_ETOOBIG;  // so many long rows: the general plan's windows
   const long long nt = (long long)L->tile.size() / 4;
   L->n_tiles = (int)nt;
   for (int c = 1; c < kWarpClasses + 2; ++c) L->class_tile_off[c] = (int)nt;
   L->Od = od;
   L->code.resize(od);
+  L->code4.resize(od - L->occ4);
   L->ref.resize(od);
   L->csr.resize(od);
   L->var.resize(od);
@@ -778,10 +792,12 @@ int build_direct_layout(const HostBDDs &H, DirectLayout *L, const int *var_deg) 
   parallel_for(nt, 64, [&](long long t0, long long t1) {
     for (long long t = t0; t < t1; ++t) {
       const long long o0 = L->tile[4 * t];
-      const int b0 = L->tile[4 * t + 1], cb_n = L->tile[4 * t + 2], depth = L->tile[4 * t + 3];
+      const int b0 = L->tile[4 * t + 1], cb_n = L->tile[4 * t + 2] & kTileCount, depth = L->tile[4 * t + 3];
+      const bool is4 = L->tile[4 * t + 2] & kTileFour;
       bool deep = depth > kLaneRegDepth;
       bool chain = L->bdd_depth[b0 + cb_n - 1] == depth;
       unsigned mask = 0;
+      int chain_end = depth;  // layers 1 .. chain_end - 1 are chain layers in every BDD of the tile
       for (int q = 0; q < 32; ++q) {
         const int cb = q < cb_n ? L->bdd_perm[b0 + q] : -1;
         const int d = cb >= 0 ? H.bdd_depth[cb] : 0;
@@ -789,6 +805,7 @@ int build_direct_layout(const HostBDDs &H, DirectLayout *L, const int *var_deg) 
           const long long o = o0 + 32LL * l + q;
           if (l >= d) {  // padding: no arcs, its own place for its difference
             L->code[o] = kDirectPad;
+            if (is4) L->code4[o - L->occ4] = kDirectPad4;
             L->ref[o] = (int)o;
             L->csr[o] = -1;
             L->var[o] = -1;
@@ -796,6 +813,21 @@ int build_direct_layout(const HostBDDs &H, DirectLayout *L, const int *var_deg) 
           }
           const long long co = H.bdd_occ0[cb] + l, cn = H.occ_node0[co];
           const bool last = l + 1 == d;
+          if (is4) {
+            unsigned c4 = 0;
+            for (int q4 = 0; q4 < 4; ++q4) {
+              auto arc4 = [&](int x) { return x == kBot ? kDirectBot4 : arc(x, last); };
+              const unsigned a = q4 < H.occ_width[co] ? arc4(H.lo[cn + q4]) | arc4(H.hi[cn + q4]) << 3 : kDirectNone4;
+              if (q4 < H.occ_width[co] && a == kDirectNone4) bad.store(true);
+              c4 |= a << (6 * q4);
+            }
+            L->code4[o - L->occ4] = c4;
+            L->code[o] = 0;
+            L->csr[o] = H.occ_csr[co];
+            L->var[o] = H.occ_var[co];
+            L->occ_of_canon[co] = (int)o;
+            continue;
+          }
           unsigned code = arc(H.lo[cn], last) | arc(H.hi[cn], last) << 2;
           if (H.occ_width[co] == 2) {
             const unsigned c1 = arc(H.lo[cn + 1], last) | arc(H.hi[cn + 1], last) << 2;
@@ -811,10 +843,16 @@ int build_direct_layout(const HostBDDs &H, DirectLayout *L, const int *var_deg) 
           deep |= var_deg[H.occ_var[co]] > 8;
           if (l < kLaneRegDepth && var_deg[H.occ_var[co]] > 2) mask |= 1u << l;
           if (l > 0 && !last && code != kDirectChain) chain = false;
+          if (l > 0 && (last || code != kDirectChain)) chain_end = std::min(chain_end, l);
         }
       }
+      if (deep) mask = (unsigned)chain_end;
       L->tile[4 * t + 3] |= (int)(mask << kTileMaskShift) | (chain ? kTileChain : 0);
       if (!chain || deep) all_chains.store(false);
+      if (is4) {
+        all_chains.store(false);
+        continue;
+      }
       if (deep) {
         L->tile[4 * t + 2] |= kTileDeep;
         int seen = deep_depth.load();

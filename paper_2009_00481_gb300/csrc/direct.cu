@@ -1,7 +1,7 @@
 // Sweeps of the direct plan (see DirectLayout in internal.h): plain min-sum solvers whose sweeps form
 // the pending shares themselves, so that an iteration is two kernels and nothing between them.
 //
-// Lane tiles: one lane per BDD of width <= 2, 32 BDDs per warp.  A warp loads its tile's
+// Lane tiles: one lane per BDD of width <= 2 (or <= 4: deep_walk4), 32 BDDs per warp.  A warp loads its tile's
 // multipliers, lane codes and differences at once (a rectangle: the addresses follow from the
 // tile's first occurrence), recomputes the messages of the other direction from the multipliers,
 // and walks the layers with everything in registers (up to kLaneRegDepth layers, no variable in more
@@ -328,21 +328,64 @@ __device__ __forceinline__ void lane_tile(const DirectParams &p, const int4 &t, 
   if (!FWD && mine) p.bdd_E[BDD_IN(p, t.y + lane, p.n_bdd)] = y0;
 }
 
+// Layers of up to four nodes: the same steps on four messages (arcs of three bits, see kDirectBot4).
+struct Four {
+  float v[4];
+};
+__device__ __forceinline__ float pull4(unsigned c, int k, const Four &x) {
+  const bool b0 = c & (1u << k), b1 = c & (2u << k);
+  const float lo = b0 ? x.v[1] : x.v[0], hi = b0 ? x.v[3] : x.v[2];
+  const float node = b1 ? hi : lo;
+  return c & (kDirectBot4 << k) ? inf() : node;
+}
+__device__ __forceinline__ void push4(unsigned c, int k, float v, Four &n) {
+  const unsigned to = (c >> k) & 7u;
+#pragma unroll
+  for (unsigned t = 0; t < 4; ++t) n.v[t] = fminf(n.v[t], to == t ? v : inf());
+}
+__device__ __forceinline__ Four step_back4(unsigned c, float lam, const Four &x) {
+  Four n;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) n.v[t] = fminf(pull4(c, 6 * t, x), lam + pull4(c, 6 * t + 3, x));
+  return n;
+}
+__device__ __forceinline__ Four step_on4(unsigned c, float lam, const Four &f) {
+  Four n{{inf(), inf(), inf(), inf()}};
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    push4(c, 6 * t, f.v[t], n);
+    push4(c, 6 * t + 3, f.v[t] + lam, n);
+  }
+  return n;
+}
+__device__ __forceinline__ float2 layer_mm4(unsigned c, float lam, const Four &f, const Four &x) {
+  float m0 = inf(), m1 = inf();
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    m0 = fminf(m0, f.v[t] + pull4(c, 6 * t, x));
+    m1 = fminf(m1, f.v[t] + lam + pull4(c, 6 * t + 3, x));
+  }
+  return make_float2(m0, m1);
+}
+
+// Deep lane tiles.  Bound by the chain of one tile: 50 frames x 200 detections of tracking (938 tiles, rows
+// of up to 97 variables) take 24 us a sweep here (31 with the arcs of every layer decoded) against
+// 35-42 us in windows of two- and four-lane teams and two pending passes of 9 and 15 us.
 // The columns of a deep lane tile in shared memory (one per lane).
 struct DeepColumns {
-  float2 *xs;
+  float2 *xs;  // (four-node tiles: float4 and, for the codes, words)
   float *lams, *shrs;
   int *refs;
   unsigned char *codes;
 };
-__device__ __forceinline__ DeepColumns deep_columns(char *smem, int depth) {
+__device__ __forceinline__ DeepColumns deep_columns(char *smem, int depth, bool four) {
   const int lane = threadIdx.x & 31;
   DeepColumns c;
-  c.xs = reinterpret_cast<float2 *>(smem) + lane;
-  c.lams = reinterpret_cast<float *>(smem + 32 * 8 * (size_t)depth) + lane;
+  c.xs = reinterpret_cast<float2 *>(smem) + (four ? 2 : 1) * lane;
+  c.lams = reinterpret_cast<float *>(smem + 32 * (four ? 16 : 8) * (size_t)depth) + lane;
   c.shrs = c.lams + 32 * depth;
   c.refs = reinterpret_cast<int *>(c.shrs + 32 * depth);
-  c.codes = reinterpret_cast<unsigned char *>(c.refs - lane + 32 * depth) + lane;
+  c.codes = reinterpret_cast<unsigned char *>(c.refs - lane + 32 * depth) + (four ? 4 : 1) * lane;
   return c;
 }
 
@@ -380,12 +423,18 @@ __device__ __forceinline__ Share wide_share(const DirectParams &p, int r, const 
 // Loads of layers l0, l0 + step, ... of a deep tile into its columns: codes, then (after the wait for
 // the sweep before) multipliers and shares, two layers' groups to a round of loads.
 template <bool FWD, int MODE>
-__device__ __forceinline__ void deep_load(const DirectParams &p, const int4 &t, const DeepColumns &c, int l0, int step,
-                                          BoundPair &sum) {
+__device__ __forceinline__ void deep_load(const DirectParams &p, const int4 &t, const DeepColumns &c, bool four, int l0,
+                                          int step, BoundPair &sum) {
   const int lane = threadIdx.x & 31, D = t.w;
   const int o = (int)BDD_IN(p, t.x + lane, p.n_occ - 32 * (D - 1));
+  if (four) {
 #pragma unroll 4
-  for (int l = l0; l < D; l += step) c.codes[32 * l] = p.code[o + 32 * l];
+    for (int l = l0; l < D; l += step)
+      reinterpret_cast<unsigned *>(c.codes)[32 * l] = p.code4[o - p.occ4 + 32 * l];
+  } else {
+#pragma unroll 4
+    for (int l = l0; l < D; l += step) c.codes[32 * l] = p.code[o + 32 * l];
+  }
   pdl_wait();
   const bool bound = FWD && MODE != kDirectFolded && p.sum_bound;
   for (int l = l0; l < D; l += 2 * step) {
@@ -410,10 +459,11 @@ __device__ __forceinline__ void deep_load(const DirectParams &p, const int4 &t, 
 
 // The walks of a deep tile over its columns, by one warp.
 template <bool FWD, int MODE>
-__device__ __forceinline__ void deep_walk(const DirectParams &p, const int4 &t, const DeepColumns &c, bool chain, BoundPair &sum) {
+__device__ __forceinline__ void deep_walk(const DirectParams &p, const int4 &t, const DeepColumns &c, int chain_end,
+                                          BoundPair &sum) {
   const int lane = threadIdx.x & 31, D = t.w;
   const int o = (int)BDD_IN(p, t.x + lane, p.n_occ - 32 * (D - 1));
-  auto inner = [&](int l) { return chain && l > 0 && l < D - 1; };
+  auto inner = [&](int l) { return l > 0 && l < chain_end; };
   // messages of the other direction (FWD: of the next layer); a layer's column entries are read a
   // layer ahead, so the recurrence does not wait on shared memory
   float y0 = 0.f, y1 = inf();
@@ -488,6 +538,54 @@ __device__ __forceinline__ void deep_walk(const DirectParams &p, const int4 &t, 
     }
   }
   if (MODE == kDirectUpdate && !FWD && mine) p.bdd_E[BDD_IN(p, t.y + lane, p.n_bdd)] = y0;
+}
+
+// The walks of a tile with layers of up to four nodes.
+template <bool FWD, int MODE>
+__device__ __forceinline__ void deep_walk4(const DirectParams &p, const int4 &t, const DeepColumns &c, BoundPair &sum) {
+  const int lane = threadIdx.x & 31, D = t.w;
+  const int o = (int)BDD_IN(p, t.x + lane, p.n_occ - 32 * (D - 1));
+  float4 *xs = reinterpret_cast<float4 *>(c.xs);
+  const unsigned *codes = reinterpret_cast<const unsigned *>(c.codes);
+  const Four start{{0.f, inf(), inf(), inf()}};
+  Four y = start;
+  for (int j = 0; j < D; ++j) {
+    const int l = FWD ? D - 1 - j : j;
+    xs[32 * l] = make_float4(y.v[0], y.v[1], y.v[2], y.v[3]);
+    y = FWD ? step_back4(codes[32 * l], c.lams[32 * l], y) : step_on4(codes[32 * l], c.lams[32 * l], y);
+  }
+  const bool mine = lane < t.z;
+  if (FWD && MODE != kDirectFolded) {
+    if (p.sum_bound) sum.add(mine ? y.v[0] : 0.f);
+    if (MODE == kDirectEnergy) {
+      if (mine) p.bdd_E[BDD_IN(p, t.y + lane, p.n_bdd)] = y.v[0];
+      return;
+    }
+  }
+  y = start;
+  for (int j = 0; j < D; ++j) {
+    const int l = FWD ? j : D - 1 - j, ol = o + 32 * l;
+    const unsigned code = codes[32 * l];
+    const float4 q = xs[32 * l];
+    const Four x{{q.x, q.y, q.z, q.w}};
+    float la = c.lams[32 * l];
+    if (MODE != kDirectFolded) la += c.shrs[32 * l];
+    const float2 m = FWD ? layer_mm4(code, la, y, x) : layer_mm4(code, la, x, y);
+    if (MODE == kDirectFolded) {
+      const long long at = p.csr[ol];
+      if (at >= 0) {
+        p.out_m0[BDD_IN(p, at, p.n_csr)] = m.x;
+        p.out_m1[BDD_IN(p, at, p.n_csr)] = m.y;
+      }
+    } else {
+      const float dd = p.omega * mm_step(m.x, m.y);
+      la -= dd;
+      p.lam[ol] = la;
+      store_diff(p, c.refs[32 * l], ol, dd);
+    }
+    y = FWD ? step_on4(code, la, y) : step_back4(code, la, y);
+  }
+  if (MODE == kDirectUpdate && !FWD && mine) p.bdd_E[BDD_IN(p, t.y + lane, p.n_bdd)] = y.v[0];
 }
 
 // per-block bound partials into the trace, by one warp in a fixed order
@@ -565,13 +663,13 @@ __global__ void __launch_bounds__(kBlockThreads, CHAINS ? 6 : 3) direct_kernel(c
   if constexpr (!CHAINS) {  // the deepest tiles, a block each: its warps load the layers, its first walks them
     if ((int)blockIdx.x < p.n_coop) {
       int4 t = p.tile[blockIdx.x];
-      const bool chain = t.w & kTileChain;
-      t.z &= kTileDeep - 1;
+      const int chain_end = t.w >> kTileMaskShift;
+      t.z &= kTileCount;
       t.w &= kTileDepth;
-      const DeepColumns c = deep_columns(smem, p.deep_depth);
-      deep_load<FWD, MODE>(p, t, c, warp, kWarpsPerBlock, acc);
+      const DeepColumns c = deep_columns(smem, t.w, false);
+      deep_load<FWD, MODE>(p, t, c, false, warp, kWarpsPerBlock, acc);
       __syncthreads();
-      if (warp == 0) deep_walk<FWD, MODE>(p, t, c, chain, acc);
+      if (warp == 0) deep_walk<FWD, MODE>(p, t, c, chain_end, acc);
     }
   }
   const int other = CHAINS ? 0 : p.n_coop;  // tiles and blocks of that kind
@@ -584,14 +682,17 @@ __global__ void __launch_bounds__(kBlockThreads, CHAINS ? 6 : 3) direct_kernel(c
     if (t1.w) prefetch_tile(p, t1);
     const int kind = t.w;
     const bool chain = t.w & kTileChain;
-    const bool deep = t.z & kTileDeep;
-    t.z &= kTileDeep - 1;
+    const bool deep = t.z & kTileDeep, four = t.z & kTileFour;
+    t.z &= kTileCount;
     t.w &= kTileDepth;
     if constexpr (!CHAINS) {
       if (deep) {
-        const DeepColumns c = deep_columns(smem + (size_t)warp * p.warp_depth * kLaneLayerBytes, p.warp_depth);
-        deep_load<FWD, MODE>(p, t, c, 0, 1, acc);
-        deep_walk<FWD, MODE>(p, t, c, chain, acc);
+        const DeepColumns c = deep_columns(smem + (size_t)warp * p.warp_bytes, t.w, four);
+        deep_load<FWD, MODE>(p, t, c, four, 0, 1, acc);
+        if (four)
+          deep_walk4<FWD, MODE>(p, t, c, acc);
+        else
+          deep_walk<FWD, MODE>(p, t, c, kind >> kTileMaskShift, acc);
         t = t1;
         t1 = t2;
         continue;

@@ -277,10 +277,16 @@ constexpr int kLaneDeepDepth = 32;  // ... up to this one (and those with a vari
                                     // rows, whose longer sums would cost every tile registers) from
                                     // shared memory: kTileDeep is set in the tile's BDD count
 constexpr int kTileDeep = 64;
+constexpr int kTileFour = 128;    // layers of up to four nodes (kTileDeep too)
+constexpr int kTileCount = 63;    // the BDD count below the flags
 constexpr int kCoopDepth = 6;
+constexpr int kCoopMost = 304;     // most tiles of more than kLaneDeepDepth layers (two blocks per SM)
+constexpr int kLaneCoopDepth = 128;  // layers of at most two nodes: up to this depth where a block takes
+                                     // each tile of more than kLaneDeepDepth layers
 constexpr int kTileChain = 256;   // in a tile's last word beside its depth: all of its BDDs have that
 constexpr int kTileDepth = 255;   // depth, and chain layers (kDirectChain) between first and last
-constexpr int kTileMaskShift = 9;  // above: a bit for each of the first layers with grouped values
+constexpr int kTileMaskShift = 9;  // above: a bit for each of the first layers with grouped values; deep
+                                   // tiles: the first layer after 0 that is not a chain layer in every BDD
 // lane codes of the direct plan: an arc (2 bits, as in lane_code) is 0 or 1 (that node of the next
 // layer; 0 also for top, which only a last layer's arcs reach) or kDirectBot
 constexpr unsigned kDirectBot = 2;
@@ -290,6 +296,12 @@ constexpr unsigned char kDirectPad = 0xA8;  // padding: node 0's 0-arc to node 0
 constexpr unsigned kDirectChain = 0u | 1u << 2 | 1u << 4 | kDirectBot << 6;
 // shared memory per layer of a deep lane tile: two messages, multiplier, share, ref, code per lane
 constexpr int kLaneLayerBytes = 32 * (8 + 4 + 4 + 4 + 1);
+// ... of one with up to four nodes a layer: four messages, a word of code
+constexpr int kLane4LayerBytes = 32 * (16 + 4 + 4 + 4 + 4);
+// codes of those: arc a of node t in bits 6 t + 3 a .. + 2 -- 0..3 (0 also for top) or kDirectBot4
+constexpr unsigned kDirectBot4 = 4;
+constexpr unsigned kDirectNone4 = kDirectBot4 | kDirectBot4 << 3;  // both arcs to bot: no such node
+constexpr unsigned kDirectPad4 = 0u | kDirectBot4 << 3 | kDirectNone4 << 6 | kDirectNone4 << 12 | kDirectNone4 << 18;
 
 struct DirectLayout {
   hvec<int> bdd_perm, bdd_depth;  // as in Layout
@@ -298,7 +310,11 @@ struct DirectLayout {
   int n_tiles = 0;
   long long Od = 0;   // occurrences with padding
   long long ext = 0;  // grouped values
-  int deep_depth = 0;  // deepest tile with kTileDeep
+  int deep_depth = 0;  // deepest tile with kTileDeep of two-node layers
+  int four_depth = 0;  // deepest tile with kTileFour
+  int n_coop = 0;      // leading tiles that need a block each (more than kLaneDeepDepth layers)
+  long long occ4 = 0;  // first occurrence of the tiles with kTileFour (the last tiles)
+  hvec<unsigned> code4;  // [Od - occ4] their codes
   bool chains = false;  // every tile has kTileChain and not kTileDeep
   hvec<unsigned char> code;  // [Od] lane codes (padding: no arcs)
   hvec<int> ref;             // [Od]
@@ -321,6 +337,8 @@ struct DirectParams {
   const int4 *tile;
   int n_tiles;
   const unsigned char *code;
+  const unsigned *code4;  // of occurrences from occ4 on
+  int occ4;
   const int *ref;
   const long long *csr;
   float *lam;
@@ -334,7 +352,7 @@ struct DirectParams {
   int deep_depth;     // deepest tile with kTileDeep, 0: none
   int chains;         // every tile is a chain tile that runs in registers
   int n_coop;         // the first n_coop tiles take a block each (all of them kTileDeep)
-  int warp_depth;     // layers of shared memory per warp of the other blocks
+  int coop_bytes, warp_bytes;  // shared memory of such a block, of a warp of the other blocks
   float omega;
   float *bdd_E;
   float *out_m0, *out_m1;  // folded pass

@@ -3,8 +3,8 @@ no pending passes between them) against the general plan, which an explicit layo
 Both run the same operations on the same values, so multipliers, pending sums and min-marginals are
 bit-identical and the bounds differ at most in the order of their FP64 sums (1e-12).  The cases sit
 at the edges of the forms an instance can take: variables in 1, 2, 3..8, 9..16, 17..32 and more rows
-(each its own way to a share), tiles of every register depth and the first deep ones, chain and
-other layers, tiles of mixed depth, rows with zero coefficients and variables in no row."""
+(each its own way to a share), tiles of every register depth and the deep ones, chain and other layers,
+layers of up to four nodes, tiles of mixed depth, rows with zero coefficients and variables in no row."""
 from __future__ import annotations
 
 import numpy as np
@@ -19,8 +19,13 @@ ITERS = 19  # graphs of 8 iterations and a ragged tail
 
 
 def rows_of(kind, cols):
-    """One row over `cols`: at most one, exactly one, a flow row, at least one."""
+    """One row over `cols`: at most one, exactly one, a flow row, at least one; layers of three and four
+    nodes: children (some count twice, at most two), at most / exactly three."""
     ones = np.ones(len(cols), np.int64)
+    if kind == "children":
+        return (cols, 1 + (np.arange(len(cols)) >= len(cols) // 3), 2, SENSE_LE)
+    if kind in ("three", "exactly_three"):
+        return (cols, ones, 3, SENSE_LE if kind == "three" else SENSE_EQ)
     if kind == "flow":
         return (cols, np.concatenate([[-1], ones[1:]]), 0, SENSE_EQ)
     return (cols, ones, 1, {"most": SENSE_LE, "one": SENSE_EQ, "least": SENSE_GE}[kind])
@@ -104,6 +109,22 @@ def test_tile_depths(cuda_lib, depth, kind):
 @pytest.mark.parametrize("depths", [[1, 2, 3, 5, 8, 10], [6, 7, 13, 20, 32], [9, 10, 11]])
 def test_mixed_depths_in_a_tile(cuda_lib, depths):
     same(instance(5, depths, ["one", "flow", "most", "least"], rows_per_depth=7))
+
+
+@pytest.mark.parametrize("depth", [6, 7, 11, 31, 32, 33])
+@pytest.mark.parametrize("kind", ["children", "three", "exactly_three"])
+def test_four_node_layers(cuda_lib, depth, kind):
+    """Layers of up to four nodes, alone and beside narrow rows (33 layers: the general plan)."""
+    s = same(instance(3, [depth], [kind], rows_per_depth=45))
+    assert s.max_width <= 4
+    same(instance(6, [4, depth], [kind, "one"], rows_per_depth=20))
+
+
+@pytest.mark.parametrize("depth", [33, 97, 128, 129])
+def test_long_narrow_rows(cuda_lib, depth):
+    """A block per tile above 32 layers; above 128 the general plan."""
+    same(instance(2, [depth], ["flow", "least"], rows_per_depth=37))
+    same(instance(4, [3, depth, 12], ["one", "most", "flow"], rows_per_depth=9))
 
 
 @pytest.mark.parametrize("omega", [0.3, 1.0])

@@ -11,8 +11,9 @@
 // a sweep.  Warp tiles stage windows of their contiguous slab in shared memory and keep the
 // current layer's messages in registers (lane t of a T-lane team holds node t; the forward step
 // pushes along lo/hi arcs with shuffles, the backward step pulls successors' messages with one
-// shuffle each).  Block tiles (layers wider than 32 nodes) keep two layer buffers in shared
-// memory (forward step by shared-memory atomic minimum).  Forward messages are written for the
+// shuffle each).  Block tiles (layers wider than 32 nodes) run one barrier a layer up to kFastWidth
+// nodes; wider ones keep two layer buffers in shared memory (forward step by shared-memory atomic
+// minimum).  Forward messages are written for the
 // backward sweep and backward messages for the next forward sweep (Prop. 3: every message
 // stays valid for the layers not yet revisited).
 //
@@ -1527,7 +1528,7 @@ __device__ __forceinline__ void block_backward(const SweepParams &p, const Phase
 }
 
 // ---------------------------------------------------------------------------------------
-// block tiles whose layers are at most kBlockThreads nodes wide (one node per thread): the
+// block tiles of smoothed solvers (layers of at most kBlockThreads nodes, one per thread): the
 // tile's node offsets and multipliers (with the shares the sweep adds) are staged in shared
 // memory once, and each thread prefetches its node's arcs two layers ahead and, in a forward
 // update, the backward messages of their targets one layer ahead, so the layer recurrence waits
